@@ -407,7 +407,7 @@ mog_status mog_render_backward_ex(mog_ctx* ctx, const mog_batch* batch, const fl
  * batch (batch->size_mask, or all), times that bucket's render kernel alone
  * over every transform schedule (schedules 0 and 1: radix schedules of its
  * FFTs, 32 = 8*4 or 8*2*2, 64 = 8*8 or 8*4*2, 128 = 8*8*2 or 8*4*4,
- * 256 = 8*8*4 or 8*4*8; schedule 2: for 64 x 64 one warp per galaxy
+ * 256 = 16*16 under both numbers; schedule 2: for 64 x 64 one warp per galaxy
  * with the 64-point transforms in registers, for 128 x 128 8*8*2 with the
  * radix-2 pass exchanged by warp shuffles instead of shared memory) x every
  * launch shape (CTAs per SM from 1 to what fits x work-queue chunk of 1..32

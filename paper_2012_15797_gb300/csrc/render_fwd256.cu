@@ -1,4 +1,6 @@
-// Fused forward render for 256 x 256 patches (Section 2, Steps 3-8).
+// Fused forward render for 256 x 256 patches (Section 2, Steps 3-8), 16 values
+// per thread (fft16.cuh), two 256-thread CTAs per SM, one galaxy at a time per
+// CTA, 16 threads per transform.
 //
 // The half spectrum (129 x 256 complex, 264 KB) does not fit in one CTA's
 // shared memory, so the transform between the two FFT directions goes through
@@ -7,70 +9,79 @@
 // occupies exactly the bytes of those two output rows (elements below N/2 in
 // row p, the rest in row p + N/2), which only that row transform overwrites.
 //
-// 512 threads, one warp per length-256 transform, two CTAs per SM (while one
-// waits at a CTA barrier the other computes):
-//   columns   8 rounds of 16 column IFFTs (round 0, warp 0: the packed nu = 0
-//             and nu = 1/2 columns); each round's row-pair values are staged in
-//             shared memory and written as coalesced 128-byte row segments
-//   rows      8 rounds of 16 row-pair IFFTs, each warp independent: load its
+//   columns   8 rounds of 16 columns.  First pass: 16 threads per column
+//             evaluate its bins (Steps 5-6) and exchange through shared memory
+//             (two buffers, one CTA barrier per round).  Second pass: 16
+//             columns side by side per half-warp, so that the row-pair inputs,
+//             formed in the thread, are stored as 128-byte segments directly
+//   rows      8 rounds of 16 row pairs, each half-warp on its own: load the
 //             row pair's input, transform, add the real-space terms, store
 //             the two pixel rows over the input
 // The PSF spectrum (272 KB) is read from global memory (L2-resident).
 //
+// What bounds it: issue slots and latency at the 16 warps per SM that 128
+// registers a thread leave (issue 54%, shared memory 50%, FMA pipe 44%; DRAM
+// below 20%).  Against 8 values per thread (radix 8 x 8 x 4, two exchanges per
+// transform, the row-pair inputs staged through shared memory with two CTA
+// barriers per round, 512 threads at 64 registers): 129k warp instructions and
+// 18k shared-memory wavefronts per galaxy instead of 199k and 43k; the 10.6k
+// 256 x 256 galaxies of the 200k mixed workload 2.47 -> 2.00 ms (with the loss
+// 2.83 -> 2.68, Lanczos 4.09 -> 3.52, composites 2.94 -> 2.65 ms).
+//
 // Lanczos variant (LZ): the Fourier part is shifted through the phase tables
 // (the Lanczos transfer function H(nu) H(omega)); a galaxy with real-space
-// terms then gets its real-space part convolved and added in two strips of
+// terms then gets its real-space part convolved and added in strips of
 // 64 rows: the 70 rows each strip needs are evaluated and convolved along x
 // (one warp per row, neighbours by shuffle) into shared memory that the
 // transforms no longer use, then convolved along y and added to the patch.
-#include "common.cuh"
-#include "internal.h"
+#include "fwd16.cuh"
 
 namespace mog {
 
 namespace {
 
 constexpr int N = 256;
-
-// float2 offset of element c of row pair p's transform input in the patch
-__device__ __forceinline__ int zpos(int p, int c) { return (c < N / 2 ? p : p + N / 2) * (N / 2) + (c & (N / 2 - 1)); }
-constexpr int H = N / 2 + 1;
-constexpr int TPF = N / 8;       // 32: one warp per transform
-constexpr int THREADS = 512;
+constexpr int T = fft16_threads<N>();      // 16
+constexpr int THREADS = 256;
+constexpr int GROUPS = THREADS / T;        // 16 transforms at a time
 constexpr int WARPS = THREADS / 32;
-constexpr int ROUNDS = (N / 2) / WARPS;   // 8
+constexpr int ROUNDS = (N / 2) / GROUPS;   // 8
 constexpr int CTAS_PER_SM = 2;
 constexpr int LS = psf_lstride(N);
 constexpr int PSF_ELEMS = psf_spec_elems(N);
-// transform rows keep N/8 float2 beyond wstride<N>(): the Lanczos strips
-// reuse that space
-constexpr int WS = wstride<N>() + N / 8;
-// twiddle tables of passes 2 and 3, room for either radix schedule
-template <int V>
-constexpr int tw_elems() { return twiddle_elems<N, Radix<N, V>::r[1]>() + twiddle_elems<N, Radix<N, V>::r[2]>(); }
-constexpr int TWS = tw_elems<0>() > tw_elems<1>() ? tw_elems<0>() : tw_elems<1>();
 constexpr int B = bucket_of(N);
+constexpr int HALF = N / 2 + 2;            // omega = 0 .. 1/2 (padded)
+constexpr int STRIP = 64;                  // Lanczos: output rows per strip
 
-// Staging rows hold the 32 columns of a round for one row pair, padded to 33
-// so that the 32 lanes of a warp (16 row pairs each for the two column
-// halves) land on distinct banks; the mirrored array is offset by 8 float2.
-constexpr int SSTR = WARPS + 1;
-constexpr size_t off_w = 0;                                              // WARPS rows of WS float2
-constexpr size_t off_sa = off_w + sizeof(float2) * WARPS * WS;            // staging [p][SSTR]
-constexpr size_t off_sb = off_sa + sizeof(float2) * ((N / 2) * SSTR + 8); // mirrored columns
-constexpr size_t off_tw = off_sb + sizeof(float2) * (N / 2) * SSTR;
-constexpr size_t off_px = off_tw + sizeof(float2) * TWS;
-constexpr size_t off_py = off_px + sizeof(float2) * H;
-constexpr size_t off_nyq = off_py + sizeof(float2) * N;
-constexpr size_t off_rec = (off_nyq + sizeof(float2) * N + 15) & ~size_t(15);
-// two record buffers of up to two records (composites), two real-space
-// tables (one per record buffer) with room for a composite's terms
-constexpr size_t off_rt = off_rec + 4 * sizeof(GalaxyRecord);
-constexpr size_t off_bar = (off_rt + 2 * sizeof(RealTermsN<2 * RMAX>) + 15) & ~size_t(15);
-constexpr size_t SMEM = off_bar + 2 * sizeof(uint64_t);
-static_assert(CTAS_PER_SM * (SMEM + 1024) <= 228 * 1024, "two CTAs share an SM's shared memory");
-constexpr int STRIP = 64;                                                 // output rows per strip
-static_assert(sizeof(float) * (STRIP + 6) * N <= off_tw, "Lanczos strip must fit below the twiddles");
+// float2 offset of element c of row pair p's transform input in the patch
+__device__ __forceinline__ int zpos(int p, int c) { return (c < N / 2 ? p : p + N / 2) * (N / 2) + (c & (N / 2 - 1)); }
+
+// Exchange row of one transform: element (k1, i) at 17 k1 + i, conflict free
+// both ways for the 16 threads of a transform.  The columns' rows are 273
+// float2 apart (odd: the second pass reads 16 columns side by side), the
+// rows' 272 (16-byte pieces).
+constexpr int EX = T + 1;
+constexpr int CS = 16 * EX + 1, RSTR = 16 * EX;
+
+template <bool COMP>
+struct Cfg256 {
+  using RT = RealTermsN<COMP ? 2 * RMAX : RMAX>;
+  static constexpr int RECS = COMP ? 2 : 1;   // records per galaxy
+  static constexpr size_t off_w = 0;          // two buffers of 16 exchange rows; Lanczos strips
+  static constexpr size_t W_BYTES = 2 * sizeof(float2) * GROUPS * CS > sizeof(float) * (STRIP + 6) * N
+                                        ? 2 * sizeof(float2) * GROUPS * CS : sizeof(float) * (STRIP + 6) * N;
+  // per galaxy, two buffers: phases along omega and nu, the nu = 1/2 column,
+  // Fourier components; records: three
+  static constexpr size_t off_py = off_w + W_BYTES;
+  static constexpr size_t off_px = off_py + 2 * sizeof(float2) * HALF;
+  static constexpr size_t off_hn = off_px + 2 * sizeof(float2) * (N / 2);
+  static constexpr size_t off_fc = (off_hn + 2 * sizeof(float2) * HALF + 15) & ~size_t(15);
+  static constexpr size_t off_rec = off_fc + 2 * sizeof(float4) * RECS * KMAX;
+  static constexpr size_t off_rt = off_rec + 3 * RECS * sizeof(GalaxyRecord);
+  static constexpr size_t SMEM = off_rt + sizeof(RT);
+  static_assert(STRIP % 2 == 0, "rows in pairs");
+  static_assert(CTAS_PER_SM * (SMEM + 512 + 1024) <= 228 * 1024, "two CTAs share an SM's shared memory");
+};
 
 // LZ, galaxy with real-space terms: patch += Lz(R), R the real-space terms at
 // the integer offset, Lz the periodic Lanczos convolution with weights wl
@@ -78,7 +89,8 @@ static_assert(sizeof(float) * (STRIP + 6) * N <= off_tw, "Lanczos strip must fit
 // Fourier part; `strip` is shared memory of (STRIP + 6) rows.
 template <int RC>
 __device__ __forceinline__ void lanczos_real_256(const RealTermsN<RC>& rt, int nr, const float* wl, float* strip,
-                                                 float* dst, int f, int j) {
+                                                 float* dst) {
+  const int j = threadIdx.x & 31;
   const int x0 = 8 * j;
   float wx[7], wy[7];
 #pragma unroll
@@ -87,36 +99,38 @@ __device__ __forceinline__ void lanczos_real_256(const RealTermsN<RC>& rt, int n
     wy[a] = wl[8 + a];
   }
   for (int y0 = 0; y0 < N; y0 += STRIP) {
-    // rows y0 - 3 .. y0 + STRIP + 2 (mod N), convolved along x
-    for (int i = f; i < STRIP + 6; i += WARPS) {
-      const int yy = (y0 - 3 + i) & (N - 1);
-      float R[8];
+    // rows y0 - 3 .. y0 + STRIP + 2 (mod N), two at a time, convolved along x
+    for (int i = 2 * (threadIdx.x >> 5); i < STRIP + 6; i += 2 * WARPS) {
+      float2 R[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) R[u] = 0.0f;
-      real_space_run(rt, nr, (float)yy, (float)x0, R);
-      float win[14];
+      for (int u = 0; u < 8; ++u) R[u] = make_float2(0.0f, 0.0f);
+      real_space_rows(rt, nr, (float)((y0 - 3 + i) & (N - 1)), (float)((y0 - 2 + i) & (N - 1)), (float)x0, R);
 #pragma unroll
-      for (int u = 0; u < 8; ++u) win[3 + u] = R[u];
+      for (int h = 0; h < 2; ++h) {
+        float win[14];
 #pragma unroll
-      for (int a = 0; a < 3; ++a) {   // x0 - 3 + a from the lane below, x0 + 8 + a from the lane above
-        win[a] = __shfl_sync(0xffffffffu, R[5 + a], (j + 31) & 31);
-        win[11 + a] = __shfl_sync(0xffffffffu, R[a], (j + 1) & 31);
+        for (int u = 0; u < 8; ++u) win[3 + u] = h ? R[u].y : R[u].x;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {   // x0 - 3 + a from the lane below, x0 + 8 + a from the lane above
+          win[a] = __shfl_sync(0xffffffffu, h ? R[5 + a].y : R[5 + a].x, (j + 31) & 31);
+          win[11 + a] = __shfl_sync(0xffffffffu, h ? R[a].y : R[a].x, (j + 1) & 31);
+        }
+        float X[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          float acc = 0.0f;
+#pragma unroll
+          for (int a = 0; a < 7; ++a) acc = fmaf(wx[a], win[3 + u - (a - 3)], acc);
+          X[u] = acc;
+        }
+        float4* srow = reinterpret_cast<float4*>(strip + (i + h) * N + x0);
+        srow[0] = make_float4(X[0], X[1], X[2], X[3]);
+        srow[1] = make_float4(X[4], X[5], X[6], X[7]);
       }
-      float X[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        float acc = 0.0f;
-#pragma unroll
-        for (int a = 0; a < 7; ++a) acc = fmaf(wx[a], win[3 + u - (a - 3)], acc);
-        X[u] = acc;
-      }
-      float4* srow = reinterpret_cast<float4*>(strip + i * N + x0);
-      srow[0] = make_float4(X[0], X[1], X[2], X[3]);
-      srow[1] = make_float4(X[4], X[5], X[6], X[7]);
     }
     __syncthreads();
     // output rows y0 + o: sum_b wy_b X(y - b), strip rows o + 3 - b
-    for (int o = f; o < STRIP; o += WARPS) {
+    for (int o = threadIdx.x >> 5; o < STRIP; o += WARPS) {
       float acc[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u) acc[u] = 0.0f;
@@ -137,60 +151,44 @@ __device__ __forceinline__ void lanczos_real_256(const RealTermsN<RC>& rt, int n
   }
 }
 
-// V: the radix schedule of the transforms (Radix<256, V>).  LOSS: the loss
-// mode of mog_render_chi2 (render_fwd.cu): the patch receives the gradient of
-// chi^2 (and serves as the transform intermediate as it does for the model).
-// COMP: composite galaxies (mog_render_composite): a second record per
-// galaxy (p.records2), both profiles' Fourier mixtures summed on the grid
-// before the one transform, both sets of real-space terms added (with LZ,
-// shifted with the Fourier part).
-template <bool LZ, bool EIG, int V = 0, bool LOSS = false, bool COMP = false>
+// LZ: the Lanczos sub-pixel shift (records carry the integer offset and the
+// fraction): the convolution of the Fourier part is folded into the phase
+// tables, the real-space part is convolved along x, // then along y, in strips.  EIG: some PSF of the context is an eigen-PSF.
+// LOSS: the loss mode of mog_render_chi2.  COMP: composites of two profiles
+// (p.records2).
+template <bool LZ, bool EIG, bool LOSS, bool COMP>
 __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) render_fwd256_kernel(RenderParams p) {
+  using C = Cfg256<COMP>;
+  using RT = typename C::RT;
   static_assert(!(LZ && LOSS), "the loss mode renders with the phase shift");
   static_assert(!(COMP && (EIG || LOSS)), "composites: constant PSFs, plain render");
-  using RT = RealTermsN<COMP ? 2 * RMAX : RMAX>;
-  constexpr int R1 = Radix<N, V>::r[1], R2 = Radix<N, V>::r[2];
-  constexpr int TW1 = twiddle_elems<N, R1>();
-  static_assert(Radix<N, V>::P == 3, "three passes");
+  constexpr int NP = N / 2;
   constexpr float INV_N = 1.0f / N;
-  constexpr float NEGLIGIBLE_LOG2 = -40.0f;
   extern __shared__ __align__(128) unsigned char smem[];
-  float2* W = reinterpret_cast<float2*>(smem + off_w);
-  float2* SA = reinterpret_cast<float2*>(smem + off_sa);
-  float2* SB = reinterpret_cast<float2*>(smem + off_sb);
-  float2* tw1 = reinterpret_cast<float2*>(smem + off_tw);
-  float2* tw2 = tw1 + TW1;
-  float2* px = reinterpret_cast<float2*>(smem + off_px);
-  float2* py = reinterpret_cast<float2*>(smem + off_py);
-  float2* nyq = reinterpret_cast<float2*>(smem + off_nyq);
-  GalaxyRecord* rec = reinterpret_cast<GalaxyRecord*>(smem + off_rec);
-  [[maybe_unused]] GalaxyRecord* rec2 = rec + 2;   // COMP: the second record of each buffer
-  RT* rts = reinterpret_cast<RT*>(smem + off_rt);
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + off_bar);   // records
-  __shared__ int s_pos[2];
-  __shared__ float s_psf_mog[KPSF][6];
-  __shared__ int s_kpsf;
-  __shared__ float s_lzw[16];   // LZ: Lanczos weights along x [0, 7) and y [8, 15)
-  __shared__ float s_eigm[KEIG];  // eigen-PSF terms of the current galaxy
+  float2* W = reinterpret_cast<float2*>(smem + C::off_w);
+  float2* pys = reinterpret_cast<float2*>(smem + C::off_py);   // [buffer][omega N = 0 .. N/2]
+  float2* pxs = reinterpret_cast<float2*>(smem + C::off_px);   // [buffer][NP]
+  float2* hns = reinterpret_cast<float2*>(smem + C::off_hn);   // [buffer][omega N = 0 .. N/2]
+  float4* fcs = reinterpret_cast<float4*>(smem + C::off_fc);   // [buffer][RECS * KMAX]
+  GalaxyRecord* rec = reinterpret_cast<GalaxyRecord*>(smem + C::off_rec);   // [3][RECS]
+  RT& rt = *reinterpret_cast<RT*>(smem + C::off_rt);
+  __shared__ int s_first[3], s_pos[2];
+  __shared__ float s_lzw[LZ ? 2 : 1][16];   // per buffer: Lanczos weights along x [0, 7) and y [8, 15)
+  __shared__ float s_chi[LOSS ? 2 : 1][WARPS];   // each warp's sum of squared residuals
 
   const int tid = threadIdx.x;
-  const int f = tid >> 5, j = tid & 31;   // warp = transform slot, lane = thread in it
-  fill_twiddles<N, R1>(tw1, 8, tid, THREADS);
-  fill_twiddles<N, R2>(tw2, N / R2, tid, THREADS);
+  const int f = tid / T, j = tid % T;
+  float2 tw[15];
+  fft16_twiddles<N>(j, tw);
+  const int cx = (f & 1) * T;   // staged output rows, see below
   const int count = p.bucket_count[B];
-  const int first = p.bucket_start[B];   // planned position of this bucket's first galaxy
+  const int first = p.bucket_start[B];          // planned position of this bucket's first galaxy
   const unsigned char* records = p.records + (size_t)first * RECORD_BYTES;
   [[maybe_unused]] const unsigned char* records2 = COMP ? p.records2 + (size_t)first * RECORD_BYTES : nullptr;
-  // the record(s) of planned position pos into buffer b
-  auto load_records = [&](int b, int pos) {
-    if constexpr (COMP) {
-      mbar_expect_tx(&bar[b], 2 * sizeof(GalaxyRecord));
-      bulk_copy(&rec[b], records + (size_t)pos * RECORD_BYTES, sizeof(GalaxyRecord), &bar[b]);
-      bulk_copy(&rec2[b], records2 + (size_t)pos * RECORD_BYTES, sizeof(GalaxyRecord), &bar[b]);
-    } else {
-      bulk_load(&rec[b], records + (size_t)pos * RECORD_BYTES, sizeof(GalaxyRecord), &bar[b]);
-    }
-  };
+
+  // The work queue is taken by thread 0, p.chunk positions at a time with the
+  // next chunk requested one chunk ahead; a position is published three
+  // galaxies ahead.
   int q_next = 0, q_end = 0, q_ahead = 0;
   auto next_position = [&]() -> int {
     if (q_next >= q_end) {
@@ -202,321 +200,298 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) render_fwd256_kernel(Ren
     }
     return q_next++;
   };
-  if (tid == 0) {
-    mbar_init(&bar[0], 1);
-    mbar_init(&bar[1], 1);
-    q_ahead = atomicAdd(&p.queue[B], p.chunk);
-    const int p0 = next_position();
-    s_pos[0] = p0;
-    if (p0 >= 0) load_records(0, p0);
-  }
-  int cur_psf = -1, k_eig = 0;
-  const float2* psf_hat = nullptr;
-  uint32_t rec_parity = 0;
-  float2* w = W + f * WS;   // this warp's transform row
-
-  __shared__ float s_chi[WARPS];   // LOSS: each warp's sum of squared residuals
-  long long chi_gal = -1;          // thread 0: galaxy whose chi^2 is still to be written
+  // the record(s) of planned position pos into buffer b (16-byte pieces, one
+  // per thread)
+  auto load_records = [&](int b, int pos) {
+    constexpr int PIECES = sizeof(GalaxyRecord) / 16;
+    float4* const d = reinterpret_cast<float4*>(&rec[b * C::RECS]) + tid;
+    if (tid < PIECES) async_copy16(d, reinterpret_cast<const float4*>(records + (size_t)pos * RECORD_BYTES) + tid);
+    else if (COMP && tid < 2 * PIECES)
+      async_copy16(d, reinterpret_cast<const float4*>(records2 + (size_t)pos * RECORD_BYTES) + tid - PIECES);
+  };
+  // LOSS, thread 0, once every warp has added its residuals of chi_gal
+  long long chi_gal = -1;
   float chi_iv = 0.0f;
-  // thread 0, once every warp has added its residuals of galaxy chi_gal
+  int chi_buf = 0;
   auto write_chi2 = [&]() {
     if (chi_gal >= 0) {
       float t = 0.0f;
-      for (int w = 0; w < WARPS; ++w) t += s_chi[w];
+      for (int i = 0; i < WARPS; ++i) t += s_chi[chi_buf][i];
       p.chi2[chi_gal] = chi_iv * t;
       chi_gal = -1;
     }
   };
-  // No barrier at the top of the loop: a warp runs from its last row pair
-  // into the next galaxy's set-up.  Every read of the previous galaxy's
-  // tables, spectrum and staging happens before one of its column-phase
-  // barriers; its rows read only their own work row, the patch and the
-  // real-space table (one per record buffer) and the term count taken before
-  // the columns; the next barrier (record landed) precedes any write they
-  // could see.
+
+  // Tables of a galaxy.  Phases and the nu = 1/2 column are kept for omega =
+  // 0 .. 1/2: at -omega they are the complex conjugates (also the Lanczos
+  // responses, whose weights are real).  hn: the Hermitian part of the nu =
+  // 1/2 column, the mean of its value at omega and the conjugate at -omega.
+  auto shift_phase = [&](float g, float fr, const float* lzw) {
+    float2 ph;
+    sincospif(-2.0f * g * fr, &ph.y, &ph.x);
+    if constexpr (LZ) {
+      float wv[7];
+      load_weights(lzw, 0, wv);
+      ph = cmul(ph, lanczos_response(wv, fr));
+    }
+    return ph;
+  };
+  auto fourier_tables = [&](int b, const GalaxyRecord* r, int pos) {
+    if (!r->ok) return;
+    const DevPsf& ps = p.psfs[r->psf];
+    const float2* const spec = ps.spec[B];
+    const int k_eig = EIG ? ps.k_eig : 0;
+    const float* pc = p.pcoef + ((size_t)first + pos) * PCOEF;
+    const float* lzw = LZ ? p.lzw + ((size_t)first + pos) * 16 : nullptr;
+    const float gx = r->x, gy = r->y;
+    const int nf1 = r->nf, nfa = nf1 + (COMP ? r[1].nf : 0);
+    constexpr int NH = N / 2 + 1;
+    constexpr int t1 = NH, t2 = t1 + NH, t3 = t2 + NP;
+    for (int i = tid; i < t3 + nfa; i += THREADS) {
+      if (i < t1) {
+        const int l = i;
+        const float om = (float)l * INV_N;
+        float2 val[2];
+        const float2 phx = shift_phase(gx, 0.5f, lzw), phy = shift_phase(gy, om, LZ ? lzw + 8 : nullptr);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {   // at omega and -omega; N/2 is one bin, omega = -1/2
+          const float o = (h || l == N / 2) ? -om : om;
+          float acc = 0.0f;
+#pragma unroll
+          for (int u = 0; u < C::RECS; ++u) {
+            const GalaxyRecord& rr = r[u];
+            const float q = fmaf(o, fmaf(rr.s22, o, rr.s12), 0.25f * rr.s11);
+            for (int c = 0; c < rr.nf; ++c) acc = fmaf(rr.famp[c], ex2(rr.fcoef[c] * q), acc);
+          }
+          const int e = (N / 2) * LS + (h ? (N - l) & (N - 1) : l);
+          const float2 pn = (EIG && k_eig) ? eigen_bin(spec, PSF_ELEMS, k_eig, pc, e) : __ldg(spec + e);
+          val[h] = cscale(cmul(pn, cmul(phx, (h || l == N / 2) ? conjf2(phy) : phy)), acc);
+        }
+        hns[b * HALF + l] = make_float2(0.5f * (val[0].x + val[1].x), 0.5f * (val[0].y - val[1].y));
+      } else if (i < t2) {
+        pys[b * HALF + i - t1] = shift_phase(gy, (float)(i - t1) * INV_N, LZ ? lzw + 8 : nullptr);
+      } else if (i < t3) {
+        pxs[b * NP + i - t2] = shift_phase(gx, (float)(i - t2) * INV_N, lzw);
+      } else {
+        const int c = i - t3;
+        const GalaxyRecord& rr = r[(COMP && c >= nf1) ? 1 : 0];
+        const int cc = c - (COMP && c >= nf1 ? nf1 : 0);
+        fcs[b * C::RECS * KMAX + c] = make_float4(rr.famp[cc], rr.famp[cc], rr.fcoef[cc], rr.fcoef[cc]);
+      }
+    }
+  };
+
+  if (tid == 0) {
+    q_ahead = atomicAdd(&p.queue[B], p.chunk);
+    for (int i = 0; i < 3; ++i) s_first[i] = next_position();
+  }
   __syncthreads();
-  for (int buf = 0;; buf ^= 1) {
-    const int pos = s_pos[buf];
-    if (pos < 0) break;
-    if (tid == 0) {
-      const int np = next_position();
-      s_pos[buf ^ 1] = np;
-      if (np >= 0) load_records(buf ^ 1, np);
+  int pos = s_first[0], pos1 = s_first[1], pos2 = s_first[2];
+  if (pos >= 0) load_records(0, pos);
+  if (pos1 >= 0) load_records(1, pos1);
+  async_copy_wait();
+  __syncthreads();
+  if (pos >= 0) fourier_tables(0, rec, pos);
+  __syncthreads();
+
+  // Who waits for whom.  Per galaxy i the CTA meets before its columns write
+  // (C2(i - 1): every thread has left the rows of i - 1), once in each round of
+  // columns and between its columns and its rows (C1(i)).  Before C1(i): the
+  // columns of i (reading its Fourier tables and record), the Fourier tables
+  // of i + 1 (buffer (i + 1) & 1,
+  // last read before C1(i - 1); from the record of i + 1, loaded before
+  // C1(i - 1)), after C2(i - 1) the real-space terms of i, and the record of
+  // i + 2 (the buffer of i - 1, last read before C1(i - 1)).  The rows use no
+  // record: what they need of it is in registers.
+  int b3 = 0;
+  for (int buf = 0; pos >= 0; buf ^= 1) {
+    const GalaxyRecord* const r = rec + b3 * C::RECS;
+    const int b3n = b3 == 2 ? 0 : b3 + 1;
+    const bool work = r->ok != 0;   // uniform
+    const float* pc = p.pcoef + ((size_t)first + pos) * PCOEF;
+    const DevPsf& ps = p.psfs[work ? r->psf : 0];
+    const float2* const psf_hat = ps.spec[B];
+    const int k_eig = EIG ? ps.k_eig : 0;
+    const int kp = ps.k, nrt1 = work ? r->nrc * kp : 0, nrt = nrt1 + (COMP && work ? r[1].nrc * kp : 0);
+    const int64_t off = r->off;
+    [[maybe_unused]] const int64_t gal = r->gal;
+    if (pos2 >= 0) load_records(b3n == 2 ? 0 : b3n + 1, pos2);
+    int pos3 = -1;
+    if (tid == 0) pos3 = next_position();
+    [[maybe_unused]] const float* const dat = (LOSS && work) ? (p.dptr ? p.dptr[gal] : p.data + off) : nullptr;
+    if constexpr (LOSS) {
+      // the data patch's lines, on their way to L2
+      if (work)
+        for (int i = tid; i < N * N / 32; i += THREADS) prefetch_l2(dat + 32 * i);
     }
-    const bool landed = mbar_wait(&bar[buf], (rec_parity >> buf) & 1u);
-    rec_parity ^= 1u << buf;
-    const GalaxyRecord& r = rec[buf];
-    if (landed && r.ok && r.psf != cur_psf) {
-      // eigen-PSF: the spectrum at the galaxy's position is sum_c m_c S_c,
-      // formed bin by bin where it is read; mixture weights at that position
-      const DevPsf& ps = p.psfs[r.psf];
-      const float* pc = p.pcoef + ((size_t)first + pos) * PCOEF;
-      k_eig = EIG ? ps.k_eig : 0;
-      if (tid < KPSF * 6)
-        s_psf_mog[tid / 6][tid % 6] = (k_eig > 0 && tid % 6 == 0) ? pc[8 + tid / 6] : ps.mog[tid / 6][tid % 6];
-      if (tid < KEIG) s_eigm[tid] = k_eig > 0 ? pc[tid] : 0.0f;   // pcoef is only read for eigen-PSFs
-      if (tid == 0) s_kpsf = ps.k;
-      psf_hat = ps.spec[B];
-      cur_psf = k_eig > 0 ? -1 : r.psf;
-    }
-    if (__syncthreads_or(!landed)) {
-      if (tid == 0) set_status(p.status, MOG_ERR_TIMEOUT);
-      return;
-    }
-    if constexpr (LOSS)   // every warp has stored the previous galaxy and added its residuals
-      if (tid == 0) write_chi2();
-    if (!r.ok) {
-      if constexpr (LOSS)
-        if (tid == 0) p.chi2[r.gal] = __int_as_float(0x7fc00000);   // NaN: a galaxy that is skipped
-      continue;
-    }
-    float* dst = p.out + r.off;
-    [[maybe_unused]] const float* const dat = LOSS ? (p.dptr ? p.dptr[r.gal] : p.data + r.off) : nullptr;
-    [[maybe_unused]] float* const mdl = (LOSS && p.model) ? p.model + r.off : nullptr;
-    [[maybe_unused]] const float two_iv = LOSS ? 2.0f * p.ivar[r.gal] : 0.0f;
-    [[maybe_unused]] float chi_acc = 0.0f;
-    if constexpr (LOSS)   // the data patch's lines on their way to L2 while the transforms run
-      for (int i = tid; i < N * N / 32; i += THREADS) prefetch_l2(dat + 32 * i);
+
     // row-pair inputs, [p][k]: the patch itself, or, when adding to what the
     // patch holds, this CTA's slice of the workspace scratch
-    float2* zbuf = p.accumulate ? p.scratch256 + (size_t)blockIdx.x * (N / 2) * N : reinterpret_cast<float2*>(dst);
+    float2* const zbuf = p.accumulate ? p.scratch256 + (size_t)blockIdx.x * (N / 2) * N
+                                      : reinterpret_cast<float2*>(p.out + off);
 
-    // per-galaxy tables
-    {
-      const float gx = r.x, gy = r.y;
-      const float* lzw = LZ ? p.lzw + ((size_t)first + pos) * 16 : nullptr;
-      const int kp = s_kpsf;
-      // COMP: the second profile's terms follow the first's (nrt1 of them)
-      const int nrt1 = r.nrc * kp, nrt = nrt1 + (COMP ? rec2[buf].nrc * kp : 0);
-      const int ntask = H + 2 * N + real_terms_padded(nrt);
-      for (int i = tid; i < ntask; i += THREADS) {
-        float sn, cs;
-        if (i < H) {
-          sincospif(-2.0f * gx * (float)i * INV_N, &sn, &cs);
-          float2 ph = make_float2(cs, sn);
-          if constexpr (LZ) {
-            float wv[7];
-            load_weights(lzw, 0, wv);
-            ph = cmul(ph, lanczos_response(wv, (float)i * INV_N));
-            if (i == 0)
+    // ---- Steps 5-6 on the bins l = j + m T of each of the group's columns, Step 7a ----
+    float2 v[16];
+    if (work) {
+      const float2* const py = pys + buf * HALF;
+      const float4* const fc = fcs + buf * C::RECS * KMAX;
+#pragma unroll 1
+      for (int cc = 0; cc < ROUNDS; ++cc) {
+        const int col = GROUPS * cc + f;   // column nu = col / N
+        const float2* ph = psf_hat + col * LS + j;
+        const float nu = (float)col * INV_N;
+        const float2 pxk = pxs[buf * NP + col];
+        if (!(EIG && k_eig)) {
 #pragma unroll
-              for (int u = 0; u < 7; ++u) s_lzw[u] = wv[u];
-          }
-          px[i] = ph;
-        } else if (i < H + N) {
-          const int l = i - H;
-          const float om = (float)(l < N / 2 ? l : l - N) * INV_N;
-          sincospif(-2.0f * gy * om, &sn, &cs);
-          float2 ph = make_float2(cs, sn);
-          if constexpr (LZ) {
-            float wv[7];
-            load_weights(lzw, 8, wv);
-            ph = cmul(ph, lanczos_response(wv, om));
-            if (l == 0)
-#pragma unroll
-              for (int u = 0; u < 7; ++u) s_lzw[8 + u] = wv[u];
-          }
-          py[l] = ph;
-        } else if (i < H + 2 * N) {
-          const int l = i - H - N;
-          const float om = (float)(l < N / 2 ? l : l - N) * INV_N;
-          const float q = fmaf(om, fmaf(r.s22, om, r.s12), 0.25f * r.s11);
-          float acc = 0.0f;
-          for (int c = 0; c < r.nf; ++c) acc = fmaf(r.famp[c], ex2(r.fcoef[c] * q), acc);
-          if constexpr (COMP) {
-            const GalaxyRecord& r2 = rec2[buf];
-            const float q2 = fmaf(om, fmaf(r2.s22, om, r2.s12), 0.25f * r2.s11);
-            for (int c = 0; c < r2.nf; ++c) acc = fmaf(r2.famp[c], ex2(r2.fcoef[c] * q2), acc);
-          }
-          float sy, cy;
-          sincospif(-2.0f * gy * om, &sy, &cy);
-          sincospif(-gx, &sn, &cs);
-          float2 phx = make_float2(cs, sn), phy = make_float2(cy, sy);
-          if constexpr (LZ) {
-            float wv[7];
-            load_weights(lzw, 0, wv);
-            phx = cmul(phx, lanczos_response(wv, 0.5f));
-            load_weights(lzw, 8, wv);
-            phy = cmul(phy, lanczos_response(wv, om));
-          }
-          const float2 pn = k_eig ? eigen_bin(psf_hat, PSF_ELEMS, k_eig, s_eigm, (N / 2) * LS + l)
-                                  : psf_hat[(N / 2) * LS + l];
-          nyq[l] = cscale(cmul(pn, cmul(phx, phy)), acc);
-        } else {
-          const int t = i - H - 2 * N;
-          if (t < nrt1) real_term(r, s_psf_mog, nullptr, kp, N, t, &rts[buf]);
-          else if (COMP && t < nrt) real_term(rec2[buf], s_psf_mog, nullptr, kp, N, t - nrt1, &rts[buf], t);
-          else real_term_zero(t, &rts[buf]);
+          for (int m = 0; m < 16; ++m) v[m] = __ldg(ph + m * T);
         }
-      }
-    }
-    __syncthreads();
-
-    const int nf = r.nf;
-    const float s11 = r.s11, s12x2 = 2.0f * r.s12, s22 = r.s22;
-    // the rows' term count, read while the next galaxy cannot yet change s_kpsf
-    const int nr = real_terms_padded((r.nrc + (COMP ? rec2[buf].nrc : 0)) * s_kpsf);
-    float2 v[8];
-    // ---- Steps 5-7a: columns k = 32 round + warp ----
-    for (int round = 0; round < ROUNDS; ++round) {
-      const int k = WARPS * round + f;
-      {
-        const float nu = k * INV_N;
-        const float a0 = s11 * nu * nu, a1 = s12x2 * nu;
-        float q[8], s[8];
-        float qmin = 3.4e38f;
+        float2 s[8];
 #pragma unroll
-        for (int m = 0; m < 8; ++m) {
-          const int l = j + m * TPF;
-          const float om = (float)(l < N / 2 ? l : l - N) * INV_N;
-          q[m] = fmaf(om, fmaf(s22, om, a1), a0);
-          qmin = fminf(qmin, q[m]);
-          s[m] = 0.0f;
+        for (int k = 0; k < 8; ++k) s[k] = make_float2(0.0f, 0.0f);
+        mixture16(fc, r->nf, r->s11, 2.0f * r->s12, r->s22, nu, (float)j * INV_N, s);
+        if constexpr (COMP)
+          mixture16(fc + r->nf, r[1].nf, r[1].s11, 2.0f * r[1].s12, r[1].s22, nu, (float)j * INV_N, s);
+#pragma unroll
+        for (int m = 0; m < 16; ++m) {
+          const int l = j + m * T;
+          if (EIG && k_eig) v[m] = eigen_bin(psf_hat, PSF_ELEMS, k_eig, pc, col * LS + l);
+          const float2 e = m < 8 ? cmul(pxk, py[l]) : cmulc(pxk, py[N - l]);
+          v[m] = cscale(cmul(v[m], e), (m & 1) ? s[m >> 1].y : s[m >> 1].x);
         }
-        for (int i = 0; i < nf; ++i) {
-          const float a = r.famp[i], c = r.fcoef[i];
-          if (!__any_sync(0xffffffffu, c * qmin > NEGLIGIBLE_LOG2)) continue;
+        if (col == 0) {
+          // Pack the Hermitian parts of the nu = 0 and nu = 1/2 columns as
+          // re + i im.  The nu = 0 column is Hermitian in omega by construction
+          // (its self-conjugate bin l = N/2 keeps its real part).
+          const float2* const hn = hns + buf * HALF;
 #pragma unroll
-          for (int m = 0; m < 8; ++m) s[m] = fmaf(a, ex2(c * q[m]), s[m]);
-        }
-        if constexpr (COMP) {
-          // the second profile's components, on its own quadratic form
-          const GalaxyRecord& r2 = rec2[buf];
-          const float b0 = r2.s11 * nu * nu, b1 = 2.0f * r2.s12 * nu, t22 = r2.s22;
-          float qmin2 = 3.4e38f;
-#pragma unroll
-          for (int m = 0; m < 8; ++m) {
-            const int l = j + m * TPF;
-            const float om = (float)(l < N / 2 ? l : l - N) * INV_N;
-            q[m] = fmaf(om, fmaf(t22, om, b1), b0);
-            qmin2 = fminf(qmin2, q[m]);
-          }
-          for (int i = 0; i < r2.nf; ++i) {
-            const float a = r2.famp[i], c = r2.fcoef[i];
-            if (!__any_sync(0xffffffffu, c * qmin2 > NEGLIGIBLE_LOG2)) continue;
-#pragma unroll
-            for (int m = 0; m < 8; ++m) s[m] = fmaf(a, ex2(c * q[m]), s[m]);
-          }
-        }
-        const float2 pxk = px[k];
-#pragma unroll
-        for (int m = 0; m < 8; ++m) {
-          const int l = j + m * TPF;
-          const float2 pv = k_eig ? eigen_bin(psf_hat, PSF_ELEMS, k_eig, s_eigm, k * LS + l) : __ldg(&psf_hat[k * LS + l]);
-          v[m] = cscale(cmul(pv, cmul(pxk, py[l])), s[m]);
-        }
-        if (k == 0) {
-#pragma unroll
-          for (int m = 0; m < 8; ++m) {
-            const int l = j + m * TPF;
+          for (int m = 0; m < 16; ++m) {
+            const int l = j + m * T;
             const float2 dc = (l == N / 2) ? make_float2(v[m].x, 0.0f) : v[m];
-            const float2 a = nyq[l], b = nyq[(N - l) & (N - 1)];
-            const float2 hn = make_float2(0.5f * (a.x + b.x), 0.5f * (a.y - b.y));
-            v[m] = make_float2(dc.x - hn.y, dc.y + hn.x);
+            const float2 h = m < 8 ? hn[l] : conjf2(hn[N - l]);
+            v[m] = make_float2(dc.x - h.y, dc.y + h.x);
           }
         }
-      }
-      dft8<+1>(v);
+        if (cc == 0) __syncthreads();   // C2 of the previous galaxy
+        float2* const wr = W + (cc & 1) * GROUPS * CS + f * CS + j;
+        dft16<+1>(v);
 #pragma unroll
-      for (int m = 0; m < 8; ++m) w[swz<N>(8 * j + m)] = v[m];
-      __syncwarp();
-      stockham_load<N, R1, +1>(w, j, tw1, v);
-      __syncwarp();
-      stockham_store<N, R1>(w, j, 8, v);
-      __syncwarp();
-      stockham_load<N, R2, +1>(w, j, tw2, v);
-      // rows p and p + N/2 (outputs m and m + R2/2 of this thread, p < N/2):
-      // stage Z_p[k] = A + iB and Z_p[N-k] = conj(A) + i conj(B)
-      {
-        constexpr int NS = N / R2;
+        for (int k1 = 0; k1 < 16; ++k1) wr[k1 * EX] = k1 ? cmul(v[at16(k1)], tw[k1 - 1]) : v[0];
+        __syncthreads();   // this round's first passes are done (and the reads of the round before last)
+        // second pass: thread (t, c) of column k = 16 cc + c, c along the half-warp
+        const int t = f, k = GROUPS * cc + j;
+        const float2* const rd = W + (cc & 1) * GROUPS * CS + j * CS + t * EX;
 #pragma unroll
-        for (int qq = 0; qq < 8 / R2; ++qq)
+        for (int i = 0; i < 16; ++i) v[i] = rd[i];
+        dft16<+1>(v);
+        // rows n = t + 16 k2: pairs (p, p + N/2) are k2, k2 + 8
+        float2* const zk = zbuf + zpos(t, k);
+        float2* const zm = zbuf + zpos(t, k ? N - k : N / 2);
 #pragma unroll
-          for (int m = 0; m < R2 / 2; ++m) {
-            const float2 A = v[qq * R2 + m], Bv = v[qq * R2 + m + R2 / 2];
-            const int pr = stockham_out_index<N, R2>(j, NS, qq, m);
-            if (k > 0) {
-              SA[pr * SSTR + f] = make_float2(A.x - Bv.y, A.y + Bv.x);
-              SB[pr * SSTR + f] = make_float2(A.x + Bv.y, Bv.x - A.y);
-            } else {
-              // column 0 in SA, column N/2 in SB's slot 0
-              SA[pr * SSTR] = make_float2(A.x, Bv.x);
-              SB[pr * SSTR] = make_float2(A.y, Bv.y);
-            }
-          }
-      }
-      __syncthreads();
-      // coalesced copy: row pair p gets columns 32 round + t and N - 32 round - t
-      for (int i = tid; i < (N / 2) * WARPS * 2; i += THREADS) {
-        const int pr = i / (2 * WARPS), t = i % (2 * WARPS);
-        if (t < WARPS) {
-          zbuf[zpos(pr, WARPS * round + t)] = SA[pr * SSTR + t];
-        } else {
-          const int u = t - WARPS;
-          const int col = (round == 0 && u == 0) ? N / 2 : N - WARPS * round - u;
-          zbuf[zpos(pr, col)] = SB[pr * SSTR + u];
+        for (int k2 = 0; k2 < 8; ++k2) {
+          const float2 A = v[at16(k2)], Bv = v[at16(k2 + 8)];
+          zk[16 * k2 * (N / 2)] = k ? make_float2(A.x - Bv.y, A.y + Bv.x) : make_float2(A.x, Bv.x);
+          zm[16 * k2 * (N / 2)] = k ? make_float2(A.x + Bv.y, Bv.x - A.y) : make_float2(A.y, Bv.y);
         }
       }
-      __syncthreads();
+      // the real-space terms, from the last threads down (the first ones have
+      // more of the Fourier tables)
+      const int nr2 = real_terms_padded(nrt);
+      for (int t = THREADS - 1 - tid; t < nr2; t += THREADS) {
+        if (t < nrt1) real_term(r[0], ps.mog, (EIG && k_eig) ? pc + 8 : nullptr, kp, N, t, &rt);
+        else if (COMP && t < nrt) real_term(r[1], ps.mog, nullptr, kp, N, t - nrt1, &rt, t);
+        else real_term_zero(t, &rt);
+      }
+      if constexpr (LZ) {
+        if (tid < 16) s_lzw[buf][tid] = p.lzw[((size_t)first + pos) * 16 + tid];
+      }
+    } else {
+      __syncthreads();   // C2
+    }
+    if (pos1 >= 0) fourier_tables(buf ^ 1, rec + b3n * C::RECS, pos1);
+    if (tid == 0) s_pos[buf] = pos3;
+    async_copy_wait();
+    __syncthreads();   // C1
+    pos3 = s_pos[buf];
+    if constexpr (LOSS) {
+      if (tid == 0) {
+        write_chi2();   // the previous galaxy's
+        if (!work) p.chi2[gal] = __int_as_float(0x7fc00000);   // NaN: a galaxy that is skipped
+      }
     }
 
-    // ---- Step 7b + 8: row pairs p = 32 round + warp, each warp on its own ----
-    const RT& rt = rts[buf];
-    for (int round = 0; round < ROUNDS; ++round) {
-      const int pr = WARPS * round + f;
+    // ---- Step 7b: row pairs, inputs Z[k], k = j + m T; Step 8 ----
+    if (work) {
+      [[maybe_unused]] float* const mdl = (LOSS && p.model) ? p.model + off : nullptr;
+      [[maybe_unused]] const float iv = LOSS ? p.ivar[gal] : 0.0f;
+      [[maybe_unused]] float chi = 0.0f;
+#pragma unroll 1
+      for (int rr = 0; rr < ROUNDS; ++rr) {
+        const int pr = GROUPS * rr + f;   // rows pr and pr + N/2
 #pragma unroll
-      for (int m = 0; m < 8; ++m) v[m] = __ldcg(&zbuf[zpos(pr, j + m * TPF)]);
-      dft8<+1>(v);
-      __syncwarp();
+        for (int m = 0; m < 16; ++m) v[m] = __ldcg(&zbuf[zpos(pr, j + m * T)]);
+        float2* const w = W + f * RSTR;
+        __syncwarp();   // the group's two rows of the round before have been stored
+        fft16<N, +1>(
+            tw, v, [&](int k1) { return w + k1 * EX + j; }, [&](int q, int i) { return w + j * EX + i; });
+        // Pixel x is staged at x ^ cx ^ 4 [bit 5 of x]: the scalar stores of the
+        // warp's two groups take different banks, and so do the lanes that
+        // read runs of 8 pixels as two 16-byte pieces.
+        float* const orow = reinterpret_cast<float*>(w);
+        float* const ob[4] = {orow + (j ^ cx), orow + (j ^ cx ^ 4), orow + (j ^ cx ^ T), orow + (j ^ cx ^ T ^ 4)};
 #pragma unroll
-      for (int m = 0; m < 8; ++m) w[swz<N>(8 * j + m)] = v[m];
-      __syncwarp();
-      stockham_load<N, R1, +1>(w, j, tw1, v);
-      __syncwarp();
-      stockham_store<N, R1>(w, j, 8, v);
-      __syncwarp();
-      stockham_load<N, R2, +1>(w, j, tw2, v);
-      __syncwarp();
-      {
-        constexpr int NS = N / R2;
-        float* orow = reinterpret_cast<float*>(w);
-#pragma unroll
-        for (int qq = 0; qq < 8 / R2; ++qq)
-#pragma unroll
-          for (int m = 0; m < R2; ++m) {
-            const int n = stockham_out_index<N, R2>(j, NS, qq, m);
-            orow[n] = v[qq * R2 + m].x;
-            orow[N + n] = v[qq * R2 + m].y;
+        for (int k2 = 0; k2 < T; ++k2) {
+          const int K = 16 * k2;
+          float* const d = ob[((K >> 5) & 1) + 2 * (k2 & 1)] + (K & ~T);
+          const float2 z = v[fft16_at<N>(0, k2)];
+          d[0] = z.x;
+          d[N] = z.y;
+        }
+        __syncwarp();   // the group's two rows are complete
+        float* const dst = p.out + off + (size_t)pr * N;
+#pragma unroll 1
+        for (int i = 0; i < 2; ++i) {
+          const int x0 = 8 * (j + T * i), p0 = x0 ^ cx ^ (((x0 >> 5) & 1) << 2);
+          float2 o[8];
+          {
+            const float4 a0 = *reinterpret_cast<const float4*>(orow + p0), a1 = *reinterpret_cast<const float4*>(orow + (p0 ^ 4));
+            const float4 b0 = *reinterpret_cast<const float4*>(orow + N + p0);
+            const float4 b1 = *reinterpret_cast<const float4*>(orow + N + (p0 ^ 4));
+            o[0] = make_float2(a0.x, b0.x); o[1] = make_float2(a0.y, b0.y); o[2] = make_float2(a0.z, b0.z);
+            o[3] = make_float2(a0.w, b0.w); o[4] = make_float2(a1.x, b1.x); o[5] = make_float2(a1.y, b1.y);
+            o[6] = make_float2(a1.z, b1.z); o[7] = make_float2(a1.w, b1.w);
           }
+          if (!LZ && nrt > 0) real_space_rows(rt, nrt, (float)pr, (float)(pr + N / 2), (float)x0, o);
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            float ov[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) ov[u] = h ? o[u].y : o[u].x;
+            if constexpr (LOSS)
+              chi += loss_store8(dat, p.out + off, mdl, (int64_t)(pr + h * (N / 2)) * N + x0, ov, 2.0f * iv);
+            else store8(dst + h * (N / 2) * N + x0, ov, p.accumulate != 0);
+          }
+        }
       }
-      __syncwarp();
-      // 512 pixels (rows pr, pr + N/2), 8 consecutive per lane and step
-      for (int idx = j; idx < 2 * N / 8; idx += 32) {
-        const int h = idx / (N / 8), x0 = (idx % (N / 8)) * 8;
-        const int yy = pr + h * (N / 2);
-        const float* orow = reinterpret_cast<const float*>(w) + h * N + x0;
-        const float4 i0 = *reinterpret_cast<const float4*>(orow), i1 = *reinterpret_cast<const float4*>(orow + 4);
-        float o[8] = {i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w};
-        if (nr > 0 && !LZ) real_space_run(rt, nr, (float)yy, (float)x0, o);
-        if constexpr (LOSS) chi_acc += loss_store8(dat, dst, mdl, (int64_t)yy * N + x0, o, two_iv);
-        else store8(dst + yy * N + x0, o, p.accumulate != 0);
-      }
-      __syncwarp();
-    }
-    if constexpr (LOSS) {
-      for (int o2 = 16; o2 > 0; o2 >>= 1) chi_acc += __shfl_xor_sync(0xffffffffu, chi_acc, o2);
-      if (j == 0) s_chi[f] = chi_acc;
-      if (tid == 0) {
-        chi_gal = r.gal;
-        chi_iv = 0.5f * two_iv;
+      if constexpr (LOSS) {
+        for (int o2 = 16; o2 > 0; o2 >>= 1) chi += __shfl_xor_sync(0xffffffffu, chi, o2);
+        if ((tid & 31) == 0) s_chi[LOSS ? buf : 0][tid >> 5] = chi;
+        if (tid == 0) {
+          chi_gal = gal;
+          chi_iv = iv;
+          chi_buf = buf;
+        }
       }
     }
     if constexpr (LZ) {
-      if (nr > 0) {   // uniform over the CTA
-        __syncthreads();   // the whole Fourier part is in the patch; W, SA, SB are free
-        lanczos_real_256(rt, nr, s_lzw, reinterpret_cast<float*>(smem), dst, f, j);
+      if (nrt > 0) {   // uniform
+        __syncthreads();   // the whole Fourier part is in the patch; W is free
+        lanczos_real_256(rt, nrt, s_lzw[LZ ? buf : 0], reinterpret_cast<float*>(smem), p.out + off);
       }
     }
+    pos = pos1;
+    pos1 = pos2;
+    pos2 = pos3;
+    b3 = b3n;
   }
   if constexpr (LOSS) {
     __syncthreads();   // the last galaxy's residuals are in
@@ -526,43 +501,39 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) render_fwd256_kernel(Ren
 
 }  // namespace
 
-template <bool LZ, bool EIG, int V = 0, bool LOSS = false, bool COMP = false>
+template <bool LZ, bool EIG, bool LOSS, bool COMP>
 static int fwd256_occupancy() {
-  const int occ = kernel_occupancy(reinterpret_cast<const void*>(render_fwd256_kernel<LZ, EIG, V, LOSS, COMP>),
-                                   THREADS, SMEM);
+  const int occ = kernel_occupancy(reinterpret_cast<const void*>(render_fwd256_kernel<LZ, EIG, LOSS, COMP>), THREADS,
+                                   Cfg256<COMP>::SMEM);
   return occ < 0 ? occ : (occ < CTAS_PER_SM ? occ : CTAS_PER_SM);
 }
 
-template <bool LZ, bool EIG, int V = 0, bool LOSS = false, bool COMP = false>
+template <bool LZ, bool EIG, bool LOSS = false, bool COMP = false>
 static cudaError_t launch_fwd256(const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s) {
-  const int occ = fwd256_occupancy<LZ, EIG, V, LOSS, COMP>();
+  const int occ = fwd256_occupancy<LZ, EIG, LOSS, COMP>();
   if (occ < 0) return cudaErrorInvalidConfiguration;
   // the accumulate mode's scratch holds one slice per CTA, CTAS_PER_SM per SM
   const int ctas = (ctas_per_sm > 0 && ctas_per_sm < occ) ? ctas_per_sm : occ;
-  render_fwd256_kernel<LZ, EIG, V, LOSS, COMP><<<num_sms * ctas, THREADS, SMEM, s>>>(p);
+  render_fwd256_kernel<LZ, EIG, LOSS, COMP><<<num_sms * ctas, THREADS, Cfg256<COMP>::SMEM, s>>>(p);
   return cudaGetLastError();
 }
 
 cudaError_t launch_render_fwd256_composite(const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s) {
-  return p.lanczos ? launch_fwd256<true, false, 0, false, true>(p, num_sms, ctas_per_sm, s)
-                   : launch_fwd256<false, false, 0, false, true>(p, num_sms, ctas_per_sm, s);
+  return p.lanczos ? launch_fwd256<true, false, false, true>(p, num_sms, ctas_per_sm, s)
+                   : launch_fwd256<false, false, false, true>(p, num_sms, ctas_per_sm, s);
 }
 
-int render_fwd256_max_ctas(int sched) {
-  return sched == 1 ? fwd256_occupancy<false, false, 1>() : fwd256_occupancy<false, false, 0>();
-}
+int render_fwd256_max_ctas(int) { return fwd256_occupancy<false, false, false, false>(); }
 
-// The second radix schedule is compiled for the plain render only.
 cudaError_t launch_render_fwd256(const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s) {
-  if (p.loss)   // the first schedule, phase shift
-    return p.eigen ? launch_fwd256<false, true, 0, true>(p, num_sms, ctas_per_sm, s)
-                   : launch_fwd256<false, false, 0, true>(p, num_sms, ctas_per_sm, s);
+  if (p.loss)
+    return p.eigen ? launch_fwd256<false, true, true>(p, num_sms, ctas_per_sm, s)
+                   : launch_fwd256<false, false, true>(p, num_sms, ctas_per_sm, s);
   if (p.eigen)
     return p.lanczos ? launch_fwd256<true, true>(p, num_sms, ctas_per_sm, s)
                      : launch_fwd256<false, true>(p, num_sms, ctas_per_sm, s);
-  if (p.lanczos) return launch_fwd256<true, false>(p, num_sms, ctas_per_sm, s);
-  return p.sched == 1 ? launch_fwd256<false, false, 1>(p, num_sms, ctas_per_sm, s)
-                      : launch_fwd256<false, false, 0>(p, num_sms, ctas_per_sm, s);
+  return p.lanczos ? launch_fwd256<true, false>(p, num_sms, ctas_per_sm, s)
+                   : launch_fwd256<false, false>(p, num_sms, ctas_per_sm, s);
 }
 
 }  // namespace mog
