@@ -337,11 +337,9 @@ mog_status mog_render_backward(mog_ctx* ctx, const mog_batch* batch, const float
  *                    of the fraction d = x - n, so d/dx (d/dy) is the
  *                    derivative through the weights and the other
  *                    gradients are those of the integer-offset render for
- *                    the transposed-convolved upstream gradient.  Computed
- *                    as three adjoint passes at the integer offsets (the
- *                    upstream patches formed on the device); uses workspace
- *                    memory of three times the gradient patches' extent and
- *                    synchronises `stream` once (to read that extent).
+ *                    the transposed-convolved upstream gradient.  One pass
+ *                    (the convolutions folded into it); 128 bytes of workspace
+ *                    per galaxy, allocated on first use.
  *                    Combines with MOG_GRAD_SERSIC.
  * Other arguments and errors as mog_render_backward.
  */

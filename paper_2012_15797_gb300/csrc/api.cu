@@ -80,9 +80,7 @@ void workspace_free(Workspace* ws) {
   cudaFree(ws->lzw);
   cudaFree(ws->pcoef);
   cudaFree(ws->bwd256);
-  cudaFree(ws->lz_up);
-  cudaFree(ws->lz_aux);
-  cudaFree(ws->lz_extent);
+  cudaFree(ws->adj_lzw);
   for (int b = 0; b < NBUCKET; ++b) {
     if (ws->side[b]) cudaStreamDestroy(ws->side[b]);
     if (ws->join_ev[b]) cudaEventDestroy(ws->join_ev[b]);
@@ -493,7 +491,7 @@ mog_status render_with(mog_ctx* ctx, Workspace* ws, const mog_batch* batch, floa
 }
 
 mog_status backward_with(mog_ctx* ctx, Workspace* ws, const mog_batch* batch, const float* grad_out,
-                         float* grad_params, cudaStream_t s, bool grad_n) {
+                         float* grad_params, cudaStream_t s, bool grad_n, bool lanczos) {
   mog_status st = check_batch(ctx, batch);
   if (st != MOG_OK) return st;
   if (batch->count == 0) return MOG_OK;
@@ -503,9 +501,18 @@ mog_status backward_with(mog_ctx* ctx, Workspace* ws, const mog_batch* batch, co
   const uint32_t want = batch->size_mask ? (batch->size_mask & BWD_BUCKETS) : BWD_BUCKETS;
   if ((want & 0x8) && !ws->bwd256)
     MOG_CUDA(ctx, cudaMalloc(&ws->bwd256, render_bwd256_scratch_bytes(ctx->num_sms)));
+  if (lanczos && batch->count > ws->adj_lzw_cap) {
+    if (ws->adj_lzw) MOG_CUDA(ctx, cudaFree(ws->adj_lzw));
+    ws->adj_lzw = nullptr;
+    ws->adj_lzw_cap = 0;
+    MOG_CUDA(ctx, cudaMalloc(&ws->adj_lzw, sizeof(float) * ADJ_LW * (size_t)batch->count));
+    ws->adj_lzw_cap = batch->count;
+  }
   RenderParams p;
   if ((st = plan_batch(ctx, ws, batch, nullptr, BWD_BUCKETS, s, &p)) != MOG_OK) return st;
   p.records = ws->adj_records;
+  p.lanczos = lanczos ? 1 : 0;
+  p.lzw = ws->adj_lzw;
   p.grad_n = grad_n ? 1 : 0;
   MOG_CUDA(ctx, launch_adjoint_prep(p, batch->count, ws->adj_records, s));
   return launch_buckets(ctx, ws, batch, BWD_BUCKETS, s, [&](int n, cudaStream_t bs) {
@@ -632,71 +639,12 @@ mog_status mog_fit_psf_mixture(mog_ctx* ctx, const float* images, int count, int
   return MOG_OK;
 }
 
-// The adjoint of the Lanczos variant (lanczos_adj.cu): three upstream
-// patches formed by transposed Lanczos convolution, three adjoint passes at
-// the integer offsets, the gradients combined.
-static mog_status lanczos_backward(mog_ctx* ctx, Workspace* ws, const mog_batch* batch, const float* grad_out,
-                                   float* grad_params, cudaStream_t s, bool grad_n) {
-  mog_status st = check_batch(ctx, batch);
-  if (st != MOG_OK) return st;
-  if (batch->count == 0) return MOG_OK;
-  if (!grad_out || (reinterpret_cast<uintptr_t>(grad_out) & 15))
-    return fail(ctx, MOG_ERR_ARG, "grad_out must be 16-byte aligned");
-  if (!grad_params) return fail(ctx, MOG_ERR_ARG, "null grad_params");
-  MOG_CUDA(ctx, cudaSetDevice(ctx->device));
-  const int64_t g = batch->count;
-  const BatchView bv = view_of(batch);
-  if (!ws->lz_extent) MOG_CUDA(ctx, cudaMalloc(&ws->lz_extent, sizeof(unsigned long long)));
-  // the upstream patches share the caller's patch offsets: their extent is
-  // read back once (this call synchronises the stream there)
-  MOG_CUDA(ctx, launch_patch_extent(bv, g, ws->lz_extent, s));
-  unsigned long long extent = 0;
-  MOG_CUDA(ctx, cudaMemcpyAsync(&extent, ws->lz_extent, sizeof(extent), cudaMemcpyDeviceToHost, s));
-  MOG_CUDA(ctx, cudaStreamSynchronize(s));
-  if (extent == 0) extent = 4;
-  if (extent > ws->lz_up_cap) {
-    if (ws->lz_up) MOG_CUDA(ctx, cudaFree(ws->lz_up));
-    ws->lz_up = nullptr;
-    ws->lz_up_cap = 0;
-    MOG_CUDA(ctx, cudaMalloc(&ws->lz_up, sizeof(float) * 3 * (size_t)extent));
-    ws->lz_up_cap = extent;
-  }
-  constexpr int AUX = 2 + 7 + 6 + 6;   // integer x, y; gradients of G0 (up to 7), Hx, Hy
-  if (g > ws->lz_aux_cap) {
-    if (ws->lz_aux) MOG_CUDA(ctx, cudaFree(ws->lz_aux));
-    ws->lz_aux = nullptr;
-    ws->lz_aux_cap = 0;
-    MOG_CUDA(ctx, cudaMalloc(&ws->lz_aux, sizeof(float) * AUX * (size_t)g));
-    ws->lz_aux_cap = g;
-  }
-  float* up0 = ws->lz_up;
-  float* upx = up0 + ws->lz_up_cap;
-  float* upy = upx + ws->lz_up_cap;
-  float* xi = ws->lz_aux;
-  float* yi = xi + g;
-  float* a0 = yi + g;
-  float* ax = a0 + 7 * g;
-  float* ay = ax + 6 * g;
-  MOG_CUDA(ctx, launch_lanczos_upstream(bv, g, grad_out, up0, upx, upy, xi, yi, s));
-  mog_batch at_n = *batch;   // the galaxies at their integer offsets
-  at_n.x = xi;
-  at_n.y = yi;
-  if ((st = backward_with(ctx, ws, &at_n, up0, a0, s, grad_n)) != MOG_OK) return st;
-  if ((st = backward_with(ctx, ws, &at_n, upx, ax, s, false)) != MOG_OK) return st;
-  if ((st = backward_with(ctx, ws, &at_n, upy, ay, s, false)) != MOG_OK) return st;
-  MOG_CUDA(ctx, launch_lanczos_combine(g, batch->flux, a0, ax, ay, grad_n ? 7 : 6, grad_params, s));
-  return MOG_OK;
-}
-
 mog_status mog_render_backward_ex(mog_ctx* ctx, const mog_batch* batch, const float* grad_out, float* grad_params,
                                   void* stream, unsigned flags) {
   if (!ctx) return MOG_ERR_ARG;
   if (flags & ~(unsigned)(MOG_GRAD_SERSIC | MOG_GRAD_LANCZOS)) return fail(ctx, MOG_ERR_ARG, "unknown gradient flags");
-  if (flags & MOG_GRAD_LANCZOS)
-    return lanczos_backward(ctx, &ctx->ws, batch, grad_out, grad_params, static_cast<cudaStream_t>(stream),
-                            (flags & MOG_GRAD_SERSIC) != 0);
   return backward_with(ctx, &ctx->ws, batch, grad_out, grad_params, static_cast<cudaStream_t>(stream),
-                       (flags & MOG_GRAD_SERSIC) != 0);
+                       (flags & MOG_GRAD_SERSIC) != 0, (flags & MOG_GRAD_LANCZOS) != 0);
 }
 
 mog_status mog_render_batch_noalloc(mog_ctx* ctx, const mog_batch* batch, float* out, void* stream) {

@@ -758,9 +758,10 @@ __device__ __forceinline__ float ramp_slope(float ns) {
   return (t > 0.0f && t < 1.0f) ? 6.0f * t * (1.0f - t) : 0.0f;
 }
 
-// Executed by one full warp (lane = mixture component); writes *out.
+// Executed by one full warp (lane = mixture component); writes *out.  With
+// `lanczos` the record's offset is the integer part, as in the forward record.
 __device__ inline void adjoint_record_warp(const BatchView& b, int64_t g, int n, const DevProfile* profiles,
-                                           const DevPsf* psfs, int* status, AdjRecord* out) {
+                                           const DevPsf* psfs, int* status, bool lanczos, AdjRecord* out) {
   const int lane = threadIdx.x & 31;
   const float flux = b.flux[g], x = b.x[g], y = b.y[g], lre = b.log_re[g];
   const float e1 = b.e1[g], e2 = b.e2[g], sn = b.sersic_n[g];
@@ -853,8 +854,8 @@ __device__ inline void adjoint_record_warp(const BatchView& b, int64_t g, int n,
     out->s12 = s12;
     out->s22 = s22;
     out->flux = flux;
-    out->x = x;
-    out->y = y;
+    out->x = lanczos ? floorf(x + 0.5f) : x;
+    out->y = lanczos ? floorf(y + 0.5f) : y;
     out->e1 = e1;
     out->e2 = e2;
     out->gal = g;
@@ -1057,6 +1058,24 @@ __device__ __forceinline__ void adj_component_tables(const AdjRecord& r, int c, 
   fd[c] = make_float4(r.fdq[c], r.fdq[c], r.fdn[c], r.fdn[c]);
 }
 
+// The Lanczos adjoint's bin: w = c_k conj(G) P, (px, pxd) the phase along nu
+// times the Lanczos response of the weights and of their slopes, (py, pyd)
+// along omega.  Adds d/dx and d/dy, the values through the slopes' responses,
+// and returns z = w px py for the other sums (contract_shape).
+__device__ __forceinline__ float2 contract_shift(float2 w, float2 px, float2 pxd, float2 py, float2 pyd, float s,
+                                                 float* acc) {
+  const float2 a = cmul(w, py), b = cmul(w, pyd);
+  acc[1] = fmaf(fmaf(a.x, pxd.x, -a.y * pxd.y), s, acc[1]);
+  acc[2] = fmaf(fmaf(b.x, px.x, -b.y * px.y), s, acc[2]);
+  return cmul(a, px);
+}
+__device__ __forceinline__ void contract_shape(float zr, float nu, float om, float s, float sq, float sn, float* acc) {
+  acc[0] = fmaf(zr, s, acc[0]);
+  acc[3] = fmaf(zr, fmaf(sq * nu, nu, sn), acc[3]);
+  acc[4] = fmaf(zr, sq * 2.0f * nu * om, acc[4]);
+  acc[5] = fmaf(zr, fmaf(sq * om, om, sn), acc[5]);
+}
+
 // Adds one bin's contribution.  z = c_k conj(G) P phase; (s, sq, sn) the
 // weighted mixture sums at the bin.
 __device__ __forceinline__ void contract_bin(float2 z, float nu, float om, float s, float sq, float sn,
@@ -1067,6 +1086,48 @@ __device__ __forceinline__ void contract_bin(float2 z, float nu, float om, float
   acc[3] = fmaf(z.x, fmaf(sq * nu, nu, sn), acc[3]);
   acc[4] = fmaf(z.x, sq * 2.0f * nu * om, acc[4]);
   acc[5] = fmaf(z.x, fmaf(sq * om, om, sn), acc[5]);
+}
+
+// Lanczos weights of the adjoint, per galaxy: w along x at [0, 7), their slopes
+// dw/dd at [8, 15), the same along y at [16, 23) and [24, 31).
+constexpr int ADJ_LW = 32;
+
+// The transposed periodic Lanczos convolutions of the upstream gradient g at 8
+// consecutive pixels (x + u, y): g0 with the weights, gx (gy) with the slopes
+// along x (y).  Along y first, over the 14 columns that the run needs.
+template <int N>
+__device__ __forceinline__ void lanczos_transposed_run(const float* gp, int gstride, int y, int x, const float* lw,
+                                                       float (&g0)[8], float (&gx)[8], float (&gy)[8]) {
+  float t[14], td[14];
+#pragma unroll
+  for (int i = 0; i < 14; ++i) t[i] = td[i] = 0.0f;
+#pragma unroll 1
+  for (int b = 0; b < 7; ++b) {
+    const float* row = gp + ((y + b - 3) & (N - 1)) * gstride;
+    const float4 p0 = *reinterpret_cast<const float4*>(row + ((x - 4) & (N - 1)));
+    const float4 p1 = *reinterpret_cast<const float4*>(row + x);
+    const float4 p2 = *reinterpret_cast<const float4*>(row + x + 4);
+    const float4 p3 = *reinterpret_cast<const float4*>(row + ((x + 8) & (N - 1)));
+    const float v[14] = {p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w, p2.x, p2.y, p2.z, p2.w, p3.x, p3.y, p3.z};
+    const float w = lw[16 + b], d = lw[24 + b];
+#pragma unroll
+    for (int i = 0; i < 14; ++i) {
+      t[i] = fmaf(w, v[i], t[i]);
+      td[i] = fmaf(d, v[i], td[i]);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < 8; ++u) g0[u] = gx[u] = gy[u] = 0.0f;
+#pragma unroll
+  for (int a = 0; a < 7; ++a) {
+    const float w = lw[a], d = lw[8 + a];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      g0[u] = fmaf(w, t[u + a], g0[u]);
+      gx[u] = fmaf(d, t[u + a], gx[u]);
+      gy[u] = fmaf(w, td[u + a], gy[u]);
+    }
+  }
 }
 
 // Real-space part of the adjoint over all pixels of an N x N patch (g read
@@ -1082,20 +1143,31 @@ __device__ __forceinline__ void contract_bin(float2 z, float nu, float om, float
 // uy^2) that every derivative of the term combines are fixed by
 // M_k = sum g E u'^k, k = 0, 1, 2: the pixel loop gathers only those three.
 // WN: also the Sersic-index sum acc[6], with S = (s11, s12, s22).
-template <int N, bool WN = false>
+// LZ: the adjoint of the Lanczos-shifted model, weights lw (ADJ_LW): the terms
+// at the integer offset are differentiated against the transposed convolution
+// of g, and the x and y sums (not divided) are their values against g through
+// the weights' slopes.
+template <int N, bool WN = false, bool LZ = false>
 __device__ __forceinline__ void adj_real_space(const float* gp, int gstride, const AdjTerms& at, int nr2, int tid,
                                                int nthreads, float* acc, float s11 = 0.f, float s12 = 0.f,
-                                               float s22 = 0.f) {
+                                               float s22 = 0.f, const float* lw = nullptr) {
   if (nr2 <= 0) return;
   const float2 NEG = make_float2(-1.0f, -1.0f), TWO = make_float2(2.0f, 2.0f), ONE = make_float2(1.0f, 1.0f);
   float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f, a4 = 0.f, a5 = 0.f, a6 = 0.f;
   for (int run = tid; run < N * N / 8; run += nthreads) {
     const int pix0 = run * 8;
     const int y = pix0 / N, x = pix0 % N;
-    const float* gr = gp + y * gstride + x;
-    const float4 ga = *reinterpret_cast<const float4*>(gr);
-    const float4 gb = *reinterpret_cast<const float4*>(gr + 4);
-    const float gw[8] = {ga.x, ga.y, ga.z, ga.w, gb.x, gb.y, gb.z, gb.w};
+    float gw[8];
+    [[maybe_unused]] float gsx[8], gsy[8];
+    if constexpr (LZ) {
+      lanczos_transposed_run<N>(gp, gstride, y, x, lw, gw, gsx, gsy);
+    } else {
+      const float* gr = gp + y * gstride + x;
+      const float4 ga = *reinterpret_cast<const float4*>(gr);
+      const float4 gb = *reinterpret_cast<const float4*>(gr + 4);
+      gw[0] = ga.x; gw[1] = ga.y; gw[2] = ga.z; gw[3] = ga.w;
+      gw[4] = gb.x; gw[5] = gb.y; gw[6] = gb.z; gw[7] = gb.w;
+    }
     const float2 Y = make_float2((float)y, (float)y), X = make_float2((float)x, (float)x);
     for (int t = 0; t < nr2; t += 2) {
       const float2 qa = *reinterpret_cast<const float2*>(&at.qa[t]);
@@ -1109,6 +1181,7 @@ __device__ __forceinline__ void adj_real_space(const float* gp, int gstride, con
       float2 rr = make_float2(ex2(e1.x), ex2(e1.y));
       const float2 r8 = *reinterpret_cast<const float2*>(&at.rrr[t]);
       float2 m0 = make_float2(0.f, 0.f), m1 = m0, m2 = m0;
+      [[maybe_unused]] float2 vx = m0, vy = m0;   // LZ: sums of E against the slopes' patches
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const float c = (float)u - 3.5f;
@@ -1116,6 +1189,10 @@ __device__ __forceinline__ void adj_real_space(const float* gp, int gstride, con
         m0 = __fadd2_rn(m0, ge);
         m1 = __ffma2_rn(ge, make_float2(c, c), m1);
         m2 = __ffma2_rn(ge, make_float2(c * c, c * c), m2);
+        if constexpr (LZ) {
+          vx = __ffma2_rn(e, make_float2(gsx[u], gsx[u]), vx);
+          vy = __ffma2_rn(e, make_float2(gsy[u], gsy[u]), vy);
+        }
         if (u < 7) {
           e = __fmul2_rn(e, rr);
           rr = __fmul2_rn(rr, r8);
@@ -1133,8 +1210,8 @@ __device__ __forceinline__ void adj_real_space(const float* gp, int gstride, con
         const float mxx = fmaf(ux, mx, i11 * t1), mxy = fmaf(uy, mx, i12 * t1), myy = fmaf(uy, my, i12 * t2);
         const float bw = at.bw[tt], bwv = at.bwv[tt], brn = at.brn[tt];
         a0 = fmaf(bw, M0, a0);
-        a1 = fmaf(bw, mx, a1);
-        a2 = fmaf(bw, my, a2);
+        a1 = fmaf(bw, LZ ? (h ? vx.y : vx.x) : mx, a1);
+        a2 = fmaf(bw, LZ ? (h ? vy.y : vy.x) : my, a2);
         a3 = fmaf(bwv, 0.5f * fmaf(-i11, M0, mxx), fmaf(brn, M0, a3));
         a4 = fmaf(bwv, fmaf(-i12, M0, mxy), a4);
         a5 = fmaf(bwv, 0.5f * fmaf(-i22, M0, myy), fmaf(brn, M0, a5));
@@ -1145,7 +1222,7 @@ __device__ __forceinline__ void adj_real_space(const float* gp, int gstride, con
       }
     }
   }
-  constexpr float INV_2PI = 0.15915494309189535f;
+  constexpr float INV_2PI = LZ ? 1.0f : 0.15915494309189535f;
   acc[0] += a0;
   acc[1] += a1 * INV_2PI;
   acc[2] += a2 * INV_2PI;

@@ -21,13 +21,8 @@ struct Workspace {
   float* lzw = nullptr;                  // 16 floats per planned galaxy (Lanczos weights)
   float* pcoef = nullptr;                // PCOEF floats per planned galaxy (eigen-PSF terms)
   float2* bwd256 = nullptr;              // per-CTA scratch of the 256 x 256 adjoint
-  // adjoint of the Lanczos variant: three upstream patches (3 x extent
-  // floats) and per galaxy the integer offsets and three gradient sets
-  float* lz_up = nullptr;
-  size_t lz_up_cap = 0;                  // floats per upstream patch set
-  float* lz_aux = nullptr;
-  int64_t lz_aux_cap = 0;                // galaxies
-  unsigned long long* lz_extent = nullptr;
+  float* adj_lzw = nullptr;              // adjoint of the Lanczos variant: ADJ_LW floats per planned galaxy
+  int64_t adj_lzw_cap = 0;               // galaxies
   cudaStream_t side[NBUCKET] = {};
   cudaEvent_t fork_ev = nullptr;
   cudaEvent_t join_ev[NBUCKET] = {};
@@ -127,7 +122,7 @@ mog_status render_with(mog_ctx* ctx, Workspace* ws, const mog_batch* batch, floa
                        bool lanczos = false, bool add = false, const LossArgs* loss = nullptr);
 mog_status backward_with(mog_ctx* ctx, Workspace* ws, const mog_batch* batch, const float* grad_out,
                          float* grad_params, cudaStream_t s,
-                         bool grad_n = false);
+                         bool grad_n = false, bool lanczos = false);
 // The library comparator (cufft_ref.cu): spectra, cuFFT C2R and the
 // real-space add for the planned galaxies of side n in `p`.
 mog_status render_cufft(mog_ctx* ctx, const RenderParams& p, int64_t count, int n, cudaStream_t s);

@@ -23,7 +23,8 @@ struct RenderParams {
   int* status;
   int chunk;                    // queue positions taken per request
   int lanczos = 0;              // 1: sub-pixel shift by Lanczos convolution
-  float* lzw = nullptr;         // lanczos: 16 floats per planned position, weights along x [0, 7), y [8, 15)
+  float* lzw = nullptr;         // lanczos: 16 floats per planned position, weights along x [0, 7), y [8, 15);
+                                // adjoint: ADJ_LW floats, weights and slopes
   float* pcoef = nullptr;       // PCOEF floats per planned position (eigen-PSF terms and mixture weights)
   int eigen = 0;                // 1: some PSF of the context is an eigen-PSF (launch the kernels that handle it)
   int accumulate = 0;           // 1: add the model to the patch instead of writing it
@@ -77,13 +78,6 @@ int render_bwd_max_ctas(int n);
 size_t render_bwd256_scratch_bytes(int num_sms);
 cudaError_t launch_render_bwd256(const RenderParams& p, const float* grad_out, float* grad_params, float2* scratch,
                                  int num_sms, cudaStream_t s);
-
-// Adjoint of the Lanczos variant (lanczos_adj.cu).
-cudaError_t launch_patch_extent(const BatchView& b, int64_t count, unsigned long long* extent, cudaStream_t s);
-cudaError_t launch_lanczos_upstream(const BatchView& b, int64_t count, const float* g, float* g0, float* hx, float* hy,
-                                    float* xi, float* yi, cudaStream_t s);
-cudaError_t launch_lanczos_combine(int64_t count, const float* flux, const float* a0, const float* ax, const float* ay,
-                                   int ng, float* out, cudaStream_t s);
 
 // Allocation-free forward render (noalloc.cu): the scratch of one call lives
 // in a fixed device array; noalloc_scratch returns its address on `device`.

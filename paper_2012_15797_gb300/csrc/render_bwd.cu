@@ -24,6 +24,7 @@
 //   reduce    warp shuffles, then one thread applies the chain rule
 #include "common.cuh"
 #include "internal.h"
+#include "lanczos_adj.cuh"
 
 namespace mog {
 
@@ -35,7 +36,9 @@ namespace mog {
 // CTA barrier.
 // WN: the variant with the Sersic-index gradient (one more mixture sum per
 // bin of the nu = 1/2 column, one more partial sum per warp).
-template <int N, int CPG = 1, bool WN = false>
+// LZ: the adjoint of the Lanczos-shifted model (more tables, fewer resident
+// CTAs for the registers of the transposed convolution).
+template <int N, int CPG = 1, bool WN = false, bool LZ = false>
 struct BwdCfg {
   static constexpr int H = N / 2 + 1;
   static constexpr int TPF = N / 8;
@@ -72,7 +75,7 @@ struct BwdCfg {
   // both would take the shared memory that the extra resident CTAs need, and
   // more resident warps hide more latency (measured: 32 x 32 1.06 -> 1.02 ms,
   // 64 x 64 2.68 -> 2.11 ms per 100k).
-  static constexpr int MIN_BLOCKS = N == 32 ? 10 : N == 64 ? 4 : CPG;
+  static constexpr int MIN_BLOCKS = LZ ? (N == 32 ? 8 : N == 64 ? 3 : 1) : N == 32 ? 10 : N == 64 ? 4 : CPG;
   // N = 64: the gradient patch and the row transforms' work rows share one
   // region (both 18 KB): the real-space pass and the row transforms' first
   // loads read the patch, then a CTA barrier, then the work rows are written
@@ -90,7 +93,10 @@ struct BwdCfg {
   static constexpr size_t off_py = off_tw + sizeof(float2) * (TW1 + TW2);
   static constexpr size_t off_nb = off_py + sizeof(float2) * N;       // nu = 1/2 column: P phase
   static constexpr size_t off_ns = off_nb + sizeof(float2) * N;       // and the mixture sums
-  static constexpr size_t off_rec = (off_ns + sizeof(float) * NYS * N + 15) & ~size_t(15);
+  // LZ: phase times slope response along omega, and the nu = 1/2 column's P
+  // phase with the slopes along x and along y
+  static constexpr size_t off_lz = (off_ns + sizeof(float) * NYS * N + 15) & ~size_t(15);
+  static constexpr size_t off_rec = off_lz + (LZ ? 3 * sizeof(float2) * N : 0);
   static constexpr size_t off_terms = off_rec + 2 * sizeof(AdjRecord);
   static constexpr size_t off_red = off_terms + sizeof(AdjTerms);
   static constexpr size_t off_bar = (off_red + sizeof(float) * RED * WARPS + 15) & ~size_t(15);
@@ -107,10 +113,14 @@ static_assert(4 * (BwdCfg<64>::SMEM + 512 + 1024) <= 196 * 1024, "64 x 64 adjoin
 // WN: also d L / d(Sersic n), a seventh gradient per galaxy.  EIG: some PSF
 // of the context is an eigen-PSF (its spectrum at the galaxy's position is
 // combined from the component spectra bin by bin where a bin is read).
-template <int N, bool WN, bool EIG, int CPG = 1>
-__global__ void __launch_bounds__(BwdCfg<N, CPG, WN>::THREADS, BwdCfg<N, CPG, WN>::MIN_BLOCKS)
+// LZ: the gradient of the Lanczos variant's model in one pass: the shift's
+// responses are folded into the phase tables, d/dx and d/dy are the values
+// through the slopes' responses, and the real-space terms (at the integer
+// offset) are contracted with the transposed convolution of the patch.
+template <int N, bool WN, bool EIG, bool LZ, int CPG = 1>
+__global__ void __launch_bounds__(BwdCfg<N, CPG, WN, LZ>::THREADS, BwdCfg<N, CPG, WN, LZ>::MIN_BLOCKS)
     render_bwd_kernel(RenderParams p, const float* __restrict__ grad_out, float* __restrict__ grad_params) {
-  using C = BwdCfg<N, CPG, WN>;
+  using C = BwdCfg<N, CPG, WN, LZ>;
   constexpr int TPF = C::TPF, WS = C::WS, LS = C::LS;
   constexpr int B = bucket_of(N);
   constexpr float INV_N = 1.0f / N;
@@ -125,6 +135,10 @@ __global__ void __launch_bounds__(BwdCfg<N, CPG, WN>::THREADS, BwdCfg<N, CPG, WN
   float2* py = reinterpret_cast<float2*>(smem + C::off_py);
   float2* nyb = reinterpret_cast<float2*>(smem + C::off_nb);
   float* nys = reinterpret_cast<float*>(smem + C::off_ns);   // [l][NYS]: S, Sq, Sn (, Sd)
+  [[maybe_unused]] float2* pyd = reinterpret_cast<float2*>(smem + C::off_lz);
+  [[maybe_unused]] float2* nybx = pyd + N;
+  [[maybe_unused]] float2* nyby = pyd + 2 * N;
+  __shared__ float s_lw[LZ ? ADJ_LW : 1];   // Lanczos weights and slopes of the current galaxy
   AdjRecord* rec = reinterpret_cast<AdjRecord*>(smem + C::off_rec);
   AdjTerms& at = *reinterpret_cast<AdjTerms*>(smem + C::off_terms);
   float* red = reinterpret_cast<float*>(smem + C::off_red);
@@ -232,6 +246,7 @@ __global__ void __launch_bounds__(BwdCfg<N, CPG, WN>::THREADS, BwdCfg<N, CPG, WN
     if (go) {
       const DevPsf& psg = p.psfs[r.psf];
       const float* pcg = p.pcoef + ((size_t)first + pos) * PCOEF;
+      [[maybe_unused]] const float* lwg = LZ ? p.lzw + ((size_t)first + pos) * ADJ_LW : nullptr;
       const float(*mog)[6] = REC_SYNC ? s_psf_mog : psg.mog;   // eigen weights in column 0 when staged
       const float* eig_w = (!REC_SYNC && k_eig > 0) ? pcg + 8 : nullptr;
       const float* eig_m = REC_SYNC ? s_eigm : pcg;
@@ -243,8 +258,17 @@ __global__ void __launch_bounds__(BwdCfg<N, CPG, WN>::THREADS, BwdCfg<N, CPG, WN
         float sn, cs;
         if (i < N) {
           const int l = i;
-          sincospif(-2.0f * gy * (float)(l < N / 2 ? l : l - N) * INV_N, &sn, &cs);
+          const float om = (float)(l < N / 2 ? l : l - N) * INV_N;
+          sincospif(-2.0f * gy * om, &sn, &cs);
           py[l] = make_float2(cs, sn);
+          if constexpr (LZ) {
+            if (l < ADJ_LW) s_lw[l] = lwg[l];
+            float w[7];
+            load_weights(lwg, 24, w);
+            pyd[l] = cmul(py[l], lanczos_response(w, om));
+            load_weights(lwg, 16, w);
+            py[l] = cmul(py[l], lanczos_response(w, om));
+          }
         } else if (i < 2 * N) {
           // the nu = 1/2 column: P phase and the mixture sums
           const int l = i - N;
@@ -263,7 +287,23 @@ __global__ void __launch_bounds__(BwdCfg<N, CPG, WN>::THREADS, BwdCfg<N, CPG, WN
           sincospif(-gx, &sn, &cs);
           const float2 pn = k_eig > 0 ? eigen_bin(psf_hat, C::PSF_ELEMS, k_eig, eig_m, (N / 2) * LS + l)
                                       : __ldg(&psf_hat[(N / 2) * LS + l]);
-          nyb[l] = cmul(pn, cmul(make_float2(cs, sn), make_float2(cy, sy)));
+          if constexpr (LZ) {
+            float w[7];
+            const float2 bx = make_float2(cs, sn), by = make_float2(cy, sy);
+            load_weights(lwg, 0, w);
+            const float2 hx = cmul(bx, lanczos_response(w, 0.5f));
+            load_weights(lwg, 8, w);
+            const float2 hxd = cmul(bx, lanczos_response(w, 0.5f));
+            load_weights(lwg, 16, w);
+            const float2 hy = cmul(by, lanczos_response(w, om));
+            load_weights(lwg, 24, w);
+            const float2 hyd = cmul(by, lanczos_response(w, om));
+            nyb[l] = cmul(pn, cmul(hx, hy));
+            nybx[l] = cmul(pn, cmul(hxd, hy));
+            nyby[l] = cmul(pn, cmul(hx, hyd));
+          } else {
+            nyb[l] = cmul(pn, cmul(make_float2(cs, sn), make_float2(cy, sy)));
+          }
           nys[C::NYS * l + 0] = s;
           nys[C::NYS * l + 1] = sq;
           nys[C::NYS * l + 2] = sn2;
@@ -298,8 +338,8 @@ __global__ void __launch_bounds__(BwdCfg<N, CPG, WN>::THREADS, BwdCfg<N, CPG, WN
     const float* gsrc = C::G_SMEM ? gbuf : grad_out + r.off;
     constexpr int GSTR = C::G_SMEM ? C::GS : N;
     if constexpr (C::ALIAS_G)   // the patch is read before the work rows overwrite it
-      adj_real_space<N, WN>(gsrc, GSTR, at, real_terms_padded(r.nrc * s_kpsf), tid, C::THREADS, acc, r.s11, r.s12,
-                            r.s22);
+      adj_real_space<N, WN, LZ>(gsrc, GSTR, at, real_terms_padded(r.nrc * s_kpsf), tid, C::THREADS, acc, r.s11, r.s12,
+                                r.s22, s_lw);
     // ---- forward FFT of row pairs (prow, prow + N/2) packed as g[prow] + i g[prow + N/2] ----
 #pragma unroll 1
     for (int rr = 0; rr < CPG; ++rr) {
@@ -339,8 +379,8 @@ __global__ void __launch_bounds__(BwdCfg<N, CPG, WN>::THREADS, BwdCfg<N, CPG, WN
 
     // ---- real-space terms: analytic derivatives, pixel by pixel ----
     if constexpr (!C::ALIAS_G)
-      adj_real_space<N, WN>(gsrc, GSTR, at, real_terms_padded(r.nrc * s_kpsf), tid, C::THREADS, acc, r.s11, r.s12,
-                            r.s22);
+      adj_real_space<N, WN, LZ>(gsrc, GSTR, at, real_terms_padded(r.nrc * s_kpsf), tid, C::THREADS, acc, r.s11, r.s12,
+                                r.s22, s_lw);
     __syncthreads();  // S3: every column input written
 
 #pragma unroll 1
@@ -372,6 +412,16 @@ __global__ void __launch_bounds__(BwdCfg<N, CPG, WN>::THREADS, BwdCfg<N, CPG, WN
         const float ck = col == 0 ? 1.0f : 2.0f;
         float2 pxf;   // e^{-2 pi i x nu}
         sincospif(-2.0f * r.x * (float)col * INV_N, &pxf.y, &pxf.x);
+        [[maybe_unused]] float2 pxd = pxf;   // LZ: times the slopes' response (pxf: the weights')
+        if constexpr (LZ) {
+          float w[7];
+#pragma unroll
+          for (int a = 0; a < 7; ++a) w[a] = s_lw[8 + a];
+          pxd = cmul(pxf, lanczos_response(w, (float)col * INV_N));
+#pragma unroll
+          for (int a = 0; a < 7; ++a) w[a] = s_lw[a];
+          pxf = cmul(pxf, lanczos_response(w, (float)col * INV_N));
+        }
         // mixture sums at the thread's bins b = q R + m, components outer and
         // bins (2k, 2k+1) in packed f32x2, BH bins per sweep over the
         // components: N = 64 takes two sweeps of 4 (its register budget at
@@ -416,13 +466,26 @@ __global__ void __launch_bounds__(BwdCfg<N, CPG, WN>::THREADS, BwdCfg<N, CPG, WN
             const float sd = (bb & 1) ? SD[bb >> 1].y : SD[bb >> 1].x;
             const float2 pv = k_eig > 0 ? eigen_bin(psf_hat, C::PSF_ELEMS, k_eig, s_eigm, col * LS + l)
                                         : __ldg(&psf_hat[col * LS + l]);
-            const float2 bph = cmul(pv, cmul(pxf, py[l]));
-            const float2 z = cscale(cmulc(bph, gk), ck);   // c_k conj(G) P phase
-            contract_bin(z, nu, om, s, sq, sn, acc);
+            float2 z;   // c_k conj(G) P phase
+            if constexpr (LZ) {
+              z = contract_shift(cscale(cmulc(pv, gk), ck), pxf, pxd, py[l], pyd[l], s, acc);
+              contract_shape(z.x, nu, om, s, sq, sn, acc);
+            } else {
+              const float2 bph = cmul(pv, cmul(pxf, py[l]));
+              z = cscale(cmulc(bph, gk), ck);
+              contract_bin(z, nu, om, s, sq, sn, acc);
+            }
             if constexpr (WN) acc[6] = fmaf(z.x, sd, acc[6]);
             if (col == 0) {
               const float2 zn = cmulc(nyb[l], gn);
-              contract_bin(zn, 0.5f, om, nys[C::NYS * l], nys[C::NYS * l + 1], nys[C::NYS * l + 2], acc);
+              if constexpr (LZ) {
+                const float sh = nys[C::NYS * l];
+                acc[1] = fmaf(fmaf(nybx[l].x, gn.x, nybx[l].y * gn.y), sh, acc[1]);
+                acc[2] = fmaf(fmaf(nyby[l].x, gn.x, nyby[l].y * gn.y), sh, acc[2]);
+                contract_shape(zn.x, 0.5f, om, sh, nys[C::NYS * l + 1], nys[C::NYS * l + 2], acc);
+              } else {
+                contract_bin(zn, 0.5f, om, nys[C::NYS * l], nys[C::NYS * l + 1], nys[C::NYS * l + 2], acc);
+              }
               if constexpr (WN) acc[6] = fmaf(zn.x, nys[C::NYS * l + 3], acc[6]);
             }
           }
@@ -448,8 +511,8 @@ __global__ void __launch_bounds__(BwdCfg<N, CPG, WN>::THREADS, BwdCfg<N, CPG, WN
       float* out = grad_params + r.gal * NACC;
       if constexpr (WN) out[6] = t[6];
       out[0] = t[0] / r.flux;
-      out[1] = TWO_PI * t[1];
-      out[2] = TWO_PI * t[2];
+      out[1] = (LZ ? 1.0f : TWO_PI) * t[1];
+      out[2] = (LZ ? 1.0f : TWO_PI) * t[2];
 #pragma unroll
       for (int k = 0; k < 3; ++k) out[3 + k] = t[3] * r.dS[k][0] + t[4] * r.dS[k][1] + t[5] * r.dS[k][2];
     }
@@ -463,33 +526,40 @@ constexpr int bwd_cpg() { return N == 128 ? 2 : 1; }
 
 static_assert(2 * (BwdCfg<128, 2, true>::SMEM + 1024) <= 228 * 1024, "two 128 x 128 adjoint CTAs share an SM");
 
-template <int N, bool WN = false, bool EIG = false>
+template <int N, bool WN = false, bool EIG = false, bool LZ = false>
 static int bwd_occupancy() {
   constexpr int CPG = bwd_cpg<N>();
-  using C = BwdCfg<N, CPG, WN>;
-  return kernel_occupancy(reinterpret_cast<const void*>(render_bwd_kernel<N, WN, EIG, CPG>), C::THREADS, C::SMEM);
+  using C = BwdCfg<N, CPG, WN, LZ>;
+  return kernel_occupancy(reinterpret_cast<const void*>(render_bwd_kernel<N, WN, EIG, LZ, CPG>), C::THREADS, C::SMEM);
 }
 
-template <int N, bool WN, bool EIG>
+template <int N, bool WN, bool EIG, bool LZ>
 static cudaError_t launch_bwd_mode(const RenderParams& p, const float* grad_out, float* grad_params, int num_sms,
                                    int ctas_per_sm, cudaStream_t s) {
   constexpr int CPG = bwd_cpg<N>();
-  using C = BwdCfg<N, CPG, WN>;
-  const int occ = bwd_occupancy<N, WN, EIG>();
+  using C = BwdCfg<N, CPG, WN, LZ>;
+  const int occ = bwd_occupancy<N, WN, EIG, LZ>();
   if (occ < 0) return cudaErrorInvalidConfiguration;
   const int ctas = (ctas_per_sm > 0 && ctas_per_sm < occ) ? ctas_per_sm : occ;
-  render_bwd_kernel<N, WN, EIG, CPG><<<ctas * num_sms, C::THREADS, C::SMEM, s>>>(p, grad_out, grad_params);
+  render_bwd_kernel<N, WN, EIG, LZ, CPG><<<ctas * num_sms, C::THREADS, C::SMEM, s>>>(p, grad_out, grad_params);
   return cudaGetLastError();
+}
+
+template <int N, bool LZ>
+static cudaError_t launch_bwd_shift(const RenderParams& p, const float* grad_out, float* grad_params, int num_sms,
+                                    int ctas_per_sm, cudaStream_t s) {
+  if (p.eigen)
+    return p.grad_n ? launch_bwd_mode<N, true, true, LZ>(p, grad_out, grad_params, num_sms, ctas_per_sm, s)
+                    : launch_bwd_mode<N, false, true, LZ>(p, grad_out, grad_params, num_sms, ctas_per_sm, s);
+  return p.grad_n ? launch_bwd_mode<N, true, false, LZ>(p, grad_out, grad_params, num_sms, ctas_per_sm, s)
+                  : launch_bwd_mode<N, false, false, LZ>(p, grad_out, grad_params, num_sms, ctas_per_sm, s);
 }
 
 template <int N>
 static cudaError_t launch_bwd(const RenderParams& p, const float* grad_out, float* grad_params, int num_sms,
                               int ctas_per_sm, cudaStream_t s) {
-  if (p.eigen)
-    return p.grad_n ? launch_bwd_mode<N, true, true>(p, grad_out, grad_params, num_sms, ctas_per_sm, s)
-                    : launch_bwd_mode<N, false, true>(p, grad_out, grad_params, num_sms, ctas_per_sm, s);
-  return p.grad_n ? launch_bwd_mode<N, true, false>(p, grad_out, grad_params, num_sms, ctas_per_sm, s)
-                  : launch_bwd_mode<N, false, false>(p, grad_out, grad_params, num_sms, ctas_per_sm, s);
+  return p.lanczos ? launch_bwd_shift<N, true>(p, grad_out, grad_params, num_sms, ctas_per_sm, s)
+                   : launch_bwd_shift<N, false>(p, grad_out, grad_params, num_sms, ctas_per_sm, s);
 }
 
 int render_bwd_max_ctas(int n) {
@@ -508,9 +578,10 @@ __global__ void adjoint_prep(RenderParams p, unsigned char* records) {
   const int warps = (gridDim.x * blockDim.x) >> 5;
   for (int pos = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; pos < total; pos += warps) {
     const int64_t g = p.order[pos];
-    adjoint_record_warp(p.b, g, p.b.size[g], p.profiles, p.psfs, p.status,
+    adjoint_record_warp(p.b, g, p.b.size[g], p.profiles, p.psfs, p.status, p.lanczos != 0,
                         reinterpret_cast<AdjRecord*>(records + (size_t)pos * sizeof(AdjRecord)));
     if (p.pcoef) eigen_coefficients_warp(p.b, g, p.psfs, p.pcoef, pos);
+    if (p.lanczos) lanczos_weights_and_slopes_warp(p.b, g, p.lzw + (size_t)pos * ADJ_LW);
   }
 }
 

@@ -49,12 +49,17 @@ constexpr size_t off_terms = off_rec + 2 * sizeof(AdjRecord);
 constexpr size_t off_red = off_terms + sizeof(AdjTerms);
 constexpr size_t off_bar = (off_red + sizeof(float) * 8 * WARPS + 15) & ~size_t(15);
 constexpr size_t SMEM = off_bar + 2 * sizeof(uint64_t);
+// LZ: phase times slope response along omega and nu, and the nu = 1/2 column's
+// P phase with the slopes along x and along y
+constexpr size_t off_lz = SMEM;
+constexpr size_t SMEM_LZ = off_lz + sizeof(float2) * (3 * N + H);
 static_assert(CTAS_PER_SM * (SMEM + 1024) <= 228 * 1024, "two CTAs share an SM's shared memory");
 
 // WN: also d L / d(Sersic n), a seventh gradient per galaxy.  EIG: some PSF of
 // the context is an eigen-PSF (its spectrum combined bin by bin where read).
-template <bool WN, bool EIG>
-__global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
+// LZ: the gradient of the Lanczos variant's model (see render_bwd.cu).
+template <bool WN, bool EIG, bool LZ>
+__global__ void __launch_bounds__(THREADS, LZ ? 1 : CTAS_PER_SM)
     render_bwd256_kernel(RenderParams p, const float* __restrict__ grad_out, float* __restrict__ grad_params,
                          float2* __restrict__ scratch_all) {
   constexpr float INV_N = 1.0f / N;
@@ -68,6 +73,11 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
   float2* py = reinterpret_cast<float2*>(smem + off_py);
   float2* nyb = reinterpret_cast<float2*>(smem + off_nb);
   float* nys = reinterpret_cast<float*>(smem + off_ns);
+  [[maybe_unused]] float2* pyd = reinterpret_cast<float2*>(smem + off_lz);
+  [[maybe_unused]] float2* nybx = pyd + N;
+  [[maybe_unused]] float2* nyby = pyd + 2 * N;
+  [[maybe_unused]] float2* pxd = pyd + 3 * N;
+  __shared__ float s_lw[LZ ? ADJ_LW : 1];   // Lanczos weights and slopes of the current galaxy
   AdjRecord* rec = reinterpret_cast<AdjRecord*>(smem + off_rec);
   AdjTerms& at = *reinterpret_cast<AdjTerms*>(smem + off_terms);
   float* red = reinterpret_cast<float*>(smem + off_red);
@@ -151,15 +161,32 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
       const int nrt = r.nrc * kp;
       const int nr2 = real_terms_padded(nrt);
       const int ntask = H + 2 * N + nr2 + r.nf;
+      [[maybe_unused]] const float* lwg = LZ ? p.lzw + ((size_t)p.bucket_start[B] + pos) * ADJ_LW : nullptr;
       for (int i = tid; i < ntask; i += THREADS) {
         float sn, cs;
         if (i < H) {
           sincospif(-2.0f * gx * (float)i * INV_N, &sn, &cs);
           px[i] = make_float2(cs, sn);
+          if constexpr (LZ) {
+            if (i < ADJ_LW) s_lw[i] = lwg[i];
+            float wv[7];
+            load_weights(lwg, 8, wv);
+            pxd[i] = cmul(px[i], lanczos_response(wv, (float)i * INV_N));
+            load_weights(lwg, 0, wv);
+            px[i] = cmul(px[i], lanczos_response(wv, (float)i * INV_N));
+          }
         } else if (i < H + N) {
           const int l = i - H;
-          sincospif(-2.0f * gy * (float)(l < N / 2 ? l : l - N) * INV_N, &sn, &cs);
+          const float om = (float)(l < N / 2 ? l : l - N) * INV_N;
+          sincospif(-2.0f * gy * om, &sn, &cs);
           py[l] = make_float2(cs, sn);
+          if constexpr (LZ) {
+            float wv[7];
+            load_weights(lwg, 24, wv);
+            pyd[l] = cmul(py[l], lanczos_response(wv, om));
+            load_weights(lwg, 16, wv);
+            py[l] = cmul(py[l], lanczos_response(wv, om));
+          }
         } else if (i < H + 2 * N) {
           const int l = i - H - N;
           const float om = (float)(l < N / 2 ? l : l - N) * INV_N;
@@ -177,7 +204,23 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
           sincospif(-gx, &sn, &cs);
           const float2 pn = k_eig > 0 ? eigen_bin(psf_hat, PSF_ELEMS, k_eig, s_eigm, (N / 2) * LS + l)
                                       : __ldg(&psf_hat[(N / 2) * LS + l]);
-          nyb[l] = cmul(pn, cmul(make_float2(cs, sn), make_float2(cy, sy)));
+          if constexpr (LZ) {
+            float wv[7];
+            const float2 bx = make_float2(cs, sn), by = make_float2(cy, sy);
+            load_weights(lwg, 0, wv);
+            const float2 hx = cmul(bx, lanczos_response(wv, 0.5f));
+            load_weights(lwg, 8, wv);
+            const float2 hxd = cmul(bx, lanczos_response(wv, 0.5f));
+            load_weights(lwg, 16, wv);
+            const float2 hy = cmul(by, lanczos_response(wv, om));
+            load_weights(lwg, 24, wv);
+            const float2 hyd = cmul(by, lanczos_response(wv, om));
+            nyb[l] = cmul(pn, cmul(hx, hy));
+            nybx[l] = cmul(pn, cmul(hxd, hy));
+            nyby[l] = cmul(pn, cmul(hx, hyd));
+          } else {
+            nyb[l] = cmul(pn, cmul(make_float2(cs, sn), make_float2(cy, sy)));
+          }
           nys[4 * l + 0] = s;
           nys[4 * l + 1] = sq;
           nys[4 * l + 2] = sn2;
@@ -237,7 +280,8 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
     }
 
     // ---- real-space terms ----
-    adj_real_space<N, WN>(gpatch, N, at, real_terms_padded(r.nrc * s_kpsf), tid, THREADS, acc, r.s11, r.s12, r.s22);
+    adj_real_space<N, WN, LZ>(gpatch, N, at, real_terms_padded(r.nrc * s_kpsf), tid, THREADS, acc, r.s11, r.s12, r.s22,
+                              s_lw);
     __syncthreads();   // scratch complete and visible
 
     // ---- columns: forward FFT along y, contraction ----
@@ -299,13 +343,25 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
           const float sn = (bb & 1) ? SN[bb >> 1].y : SN[bb >> 1].x;
           const float sd = (bb & 1) ? SD[bb >> 1].y : SD[bb >> 1].x;
           const float2 pv = k_eig > 0 ? eigen_bin(psf_hat, PSF_ELEMS, k_eig, s_eigm, k * LS + l) : __ldg(&psf_hat[k * LS + l]);
-          const float2 bph = cmul(pv, cmul(pxk, py[l]));
-          const float2 z = cscale(cmulc(bph, gk), ck);
-          contract_bin(z, nu, om, s, sq, sn, acc);
+          float2 z;
+          if constexpr (LZ) {
+            z = contract_shift(cscale(cmulc(pv, gk), ck), pxk, pxd[k], py[l], pyd[l], s, acc);
+            contract_shape(z.x, nu, om, s, sq, sn, acc);
+          } else {
+            const float2 bph = cmul(pv, cmul(pxk, py[l]));
+            z = cscale(cmulc(bph, gk), ck);
+            contract_bin(z, nu, om, s, sq, sn, acc);
+          }
           if constexpr (WN) acc[6] = fmaf(z.x, sd, acc[6]);
           if (k == 0) {
             const float2 zn = cmulc(nyb[l], gn);
-            contract_bin(zn, 0.5f, om, nys[4 * l], nys[4 * l + 1], nys[4 * l + 2], acc);
+            if constexpr (LZ) {
+              acc[1] = fmaf(fmaf(nybx[l].x, gn.x, nybx[l].y * gn.y), nys[4 * l], acc[1]);
+              acc[2] = fmaf(fmaf(nyby[l].x, gn.x, nyby[l].y * gn.y), nys[4 * l], acc[2]);
+              contract_shape(zn.x, 0.5f, om, nys[4 * l], nys[4 * l + 1], nys[4 * l + 2], acc);
+            } else {
+              contract_bin(zn, 0.5f, om, nys[4 * l], nys[4 * l + 1], nys[4 * l + 2], acc);
+            }
             if constexpr (WN) acc[6] = fmaf(zn.x, nys[4 * l + 3], acc[6]);
           }
         }
@@ -330,8 +386,8 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
       float* out = grad_params + r.gal * NACC;
       if constexpr (WN) out[6] = t[6];
       out[0] = t[0] / r.flux;
-      out[1] = TWO_PI * t[1];
-      out[2] = TWO_PI * t[2];
+      out[1] = (LZ ? 1.0f : TWO_PI) * t[1];
+      out[2] = (LZ ? 1.0f : TWO_PI) * t[2];
 #pragma unroll
       for (int c = 0; c < 3; ++c) out[3 + c] = t[3] * r.dS[c][0] + t[4] * r.dS[c][1] + t[5] * r.dS[c][2];
     }
@@ -348,12 +404,15 @@ size_t render_bwd256_scratch_bytes(int num_sms) {
 
 cudaError_t launch_render_bwd256(const RenderParams& p, const float* grad_out, float* grad_params, float2* scratch,
                                  int num_sms, cudaStream_t s) {
-  auto fn = p.eigen ? (p.grad_n ? render_bwd256_kernel<true, true> : render_bwd256_kernel<false, true>)
-                    : (p.grad_n ? render_bwd256_kernel<true, false> : render_bwd256_kernel<false, false>);
-  const int occ = kernel_occupancy(reinterpret_cast<const void*>(fn), THREADS, SMEM);
+  auto fn = p.lanczos ? (p.eigen ? (p.grad_n ? render_bwd256_kernel<true, true, true> : render_bwd256_kernel<false, true, true>)
+                                 : (p.grad_n ? render_bwd256_kernel<true, false, true> : render_bwd256_kernel<false, false, true>))
+                      : (p.eigen ? (p.grad_n ? render_bwd256_kernel<true, true, false> : render_bwd256_kernel<false, true, false>)
+                                 : (p.grad_n ? render_bwd256_kernel<true, false, false> : render_bwd256_kernel<false, false, false>));
+  const size_t smem = p.lanczos ? SMEM_LZ : SMEM;
+  const int occ = kernel_occupancy(reinterpret_cast<const void*>(fn), THREADS, smem);
   if (occ < 0) return cudaErrorInvalidConfiguration;
   // the scratch holds one slice per CTA, CTAS_PER_SM per SM
-  fn<<<num_sms * (occ < CTAS_PER_SM ? occ : CTAS_PER_SM), THREADS, SMEM, s>>>(p, grad_out, grad_params, scratch);
+  fn<<<num_sms * (occ < CTAS_PER_SM ? occ : CTAS_PER_SM), THREADS, smem, s>>>(p, grad_out, grad_params, scratch);
   return cudaGetLastError();
 }
 
