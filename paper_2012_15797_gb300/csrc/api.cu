@@ -391,16 +391,14 @@ mog_status check_batch(mog_ctx* ctx, const mog_batch* batch) {
 
 namespace {
 
-// Plans the batch on stream s and fills the launch parameters.
-mog_status plan_batch(mog_ctx* ctx, Workspace* ws, const mog_batch* batch, float* out, uint32_t supported,
-                      cudaStream_t s, RenderParams* p) {
+// Sizes the workspace for the batch and fills the launch parameters.
+mog_status batch_params(mog_ctx* ctx, Workspace* ws, const mog_batch* batch, float* out, RenderParams* p) {
   MOG_CUDA(ctx, cudaSetDevice(ctx->device));
   mog_status st = ensure_capacity(ctx, ws, batch->count);
   if (st != MOG_OK) return st;
-  const BatchView bv = view_of(batch);
-  MOG_CUDA(ctx, launch_plan(bv, batch->count, ws->plan, supported, ctx->d_status, s));
   *p = RenderParams{};
-  p->b = bv;
+  p->b = view_of(batch);
+  p->max_galaxies = batch->count;
   p->out = out;
   p->profiles = ctx->d_profiles;
   p->psfs = ctx->d_psfs;
@@ -462,12 +460,13 @@ mog_status render_with(mog_ctx* ctx, Workspace* ws, const mog_batch* batch, floa
   if (!out || (reinterpret_cast<uintptr_t>(out) & 15)) return fail(ctx, MOG_ERR_ARG, "out must be 16-byte aligned");
   const uint32_t buckets = lanczos ? LZ_BUCKETS : FWD_BUCKETS;
   const uint32_t want = batch->size_mask ? (batch->size_mask & buckets) : buckets;
-  // adding to the patch: the 256 x 256 kernel cannot use the patch as its
-  // transform intermediate, so it takes the workspace scratch
+  // adding to the patch: the 256 x 256 kernels cannot use the patch as their
+  // transform intermediate (or, with the Lanczos shift, for the Fourier part),
+  // so they take the workspace scratch
   if (add && (want & 0x8) && !ws->bwd256)
     MOG_CUDA(ctx, cudaMalloc(&ws->bwd256, render_bwd256_scratch_bytes(ctx->num_sms)));
   RenderParams p;
-  if ((st = plan_batch(ctx, ws, batch, out, buckets, s, &p)) != MOG_OK) return st;
+  if ((st = batch_params(ctx, ws, batch, out, &p)) != MOG_OK) return st;
   p.records = ws->records;
   p.lanczos = lanczos ? 1 : 0;
   p.lzw = ws->lzw;
@@ -481,7 +480,7 @@ mog_status render_with(mog_ctx* ctx, Workspace* ws, const mog_batch* batch, floa
     p.chi2 = loss->chi2;
     p.model = loss->model;
   }
-  MOG_CUDA(ctx, launch_galaxy_prep(p, batch->count, ws->records, s));
+  MOG_CUDA(ctx, launch_plan_forward(p, batch->count, ws->plan, buckets, ws->records, s));
   return launch_buckets(ctx, ws, batch, buckets, s, [&](int n, cudaStream_t bs) {
     RenderParams q = p;
     q.chunk = ctx->tune_fwd[bucket_of(n)].chunk;
@@ -509,12 +508,12 @@ mog_status backward_with(mog_ctx* ctx, Workspace* ws, const mog_batch* batch, co
     ws->adj_lzw_cap = batch->count;
   }
   RenderParams p;
-  if ((st = plan_batch(ctx, ws, batch, nullptr, BWD_BUCKETS, s, &p)) != MOG_OK) return st;
+  if ((st = batch_params(ctx, ws, batch, nullptr, &p)) != MOG_OK) return st;
   p.records = ws->adj_records;
   p.lanczos = lanczos ? 1 : 0;
   p.lzw = ws->adj_lzw;
   p.grad_n = grad_n ? 1 : 0;
-  MOG_CUDA(ctx, launch_adjoint_prep(p, batch->count, ws->adj_records, s));
+  MOG_CUDA(ctx, launch_plan_adjoint(p, batch->count, ws->plan, BWD_BUCKETS, ws->adj_records, s));
   return launch_buckets(ctx, ws, batch, BWD_BUCKETS, s, [&](int n, cudaStream_t bs) {
     RenderParams q = p;
     q.chunk = ctx->tune_bwd[bucket_of(n)].chunk;
@@ -584,14 +583,14 @@ mog_status mog_render_composite(mog_ctx* ctx, const mog_batch* first, const mog_
   // two records per galaxy: the second profile's after the first's
   if ((st = ensure_capacity(ctx, ws, 2 * g)) != MOG_OK) return st;
   RenderParams p;
-  if ((st = plan_batch(ctx, ws, first, out, FWD_BUCKETS, s, &p)) != MOG_OK) return st;
+  if ((st = batch_params(ctx, ws, first, out, &p)) != MOG_OK) return st;
   unsigned char* rec2 = ws->records + (size_t)g * RECORD_BYTES;
   p.records = ws->records;
   p.records2 = rec2;
   p.eigen = 0;   // eigen-PSF galaxies are rejected by the record prologue
   p.lanczos = (flags & MOG_RENDER_LANCZOS) ? 1 : 0;
   p.lzw = ws->lzw;
-  MOG_CUDA(ctx, launch_composite_prep(p, view_of(second), g, ws->records, rec2, s));
+  MOG_CUDA(ctx, launch_plan_composite(p, view_of(second), g, ws->plan, FWD_BUCKETS, ws->records, rec2, s));
   return launch_buckets(ctx, ws, first, FWD_BUCKETS, s, [&](int n, cudaStream_t bs) -> cudaError_t {
     RenderParams q = p;
     const LaunchShape& ls = ctx->tune_fwd[bucket_of(n)];
@@ -614,9 +613,9 @@ mog_status mog_render_batch_cufft(mog_ctx* ctx, const mog_batch* batch, float* o
   if (!cufft_available()) return fail(ctx, MOG_ERR_STATE, "the cuFFT library could not be opened");
   const cudaStream_t s = static_cast<cudaStream_t>(stream);
   RenderParams p;
-  if ((st = plan_batch(ctx, &ctx->ws, batch, out, m, s, &p)) != MOG_OK) return st;
+  if ((st = batch_params(ctx, &ctx->ws, batch, out, &p)) != MOG_OK) return st;
   p.records = ctx->ws.records;
-  MOG_CUDA(ctx, launch_galaxy_prep(p, batch->count, ctx->ws.records, s));
+  MOG_CUDA(ctx, launch_plan_forward(p, batch->count, ctx->ws.plan, m, ctx->ws.records, s));
   return render_cufft(ctx, p, batch->count, bucket_side(__builtin_ctz(m)), s);
 }
 

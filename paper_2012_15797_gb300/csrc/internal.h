@@ -22,6 +22,7 @@ struct RenderParams {
   const unsigned char* records2 = nullptr;   // composites: the second profile's record per planned position
   int* status;
   int chunk;                    // queue positions taken per request
+  int64_t max_galaxies = INT64_MAX;   // upper bound of the bucket's galaxies (the batch's count): no more CTAs
   int lanczos = 0;              // 1: sub-pixel shift by Lanczos convolution
   float* lzw = nullptr;         // lanczos: 16 floats per planned position, weights along x [0, 7), y [8, 15);
                                 // adjoint: ADJ_LW floats, weights and slopes
@@ -59,17 +60,26 @@ struct PlanScratch {
   int32_t* order;    // [capacity]
 };
 
-// Builds the bucket / PSF grouping of a batch on `s`.  `supported` is a
-// bitmask of buckets the caller can render; galaxies of other sizes are
-// reported through the status word and skipped.
-cudaError_t launch_plan(const BatchView& b, int64_t count, const PlanScratch& ps, int supported, int* status,
-                        cudaStream_t s);
+// Up to this many galaxies the plan and the records are one launch that counts
+// each galaxy's position over the batch (plan_and_records): quadratic, 2.6 us of
+// warp instructions at 2048, against three more launches of the counting sort
+// and their gaps (about 10 us).
+constexpr int64_t SMALL_PLAN = 2048;
 
-// Writes the GalaxyRecord of every planned position (Steps 3-4).
-cudaError_t launch_galaxy_prep(const RenderParams& p, int64_t count, unsigned char* records, cudaStream_t s);
+// Builds the bucket / PSF grouping of a batch (p.b) on `s` and writes the
+// record of every planned position (Steps 3-4; the adjoint's AdjRecord).
+// `supported` is a bitmask of buckets the caller can render; galaxies of other
+// sizes are reported through the status word and skipped.  Composites: the
+// first profile's records (batch p.b) at records, the second's (batch
+// `second`, same centre, size, PSF and patch) at records2.
+cudaError_t launch_plan_forward(const RenderParams& p, int64_t count, const PlanScratch& ps, int supported,
+                                unsigned char* records, cudaStream_t s);
+cudaError_t launch_plan_adjoint(const RenderParams& p, int64_t count, const PlanScratch& ps, int supported,
+                                unsigned char* records, cudaStream_t s);
+cudaError_t launch_plan_composite(const RenderParams& p, const BatchView& second, int64_t count, const PlanScratch& ps,
+                                  int supported, unsigned char* records, unsigned char* records2, cudaStream_t s);
 
-// Adjoint: records (AdjRecord per planned position) and the fused kernel.
-cudaError_t launch_adjoint_prep(const RenderParams& p, int64_t count, unsigned char* records, cudaStream_t s);
+// The adjoint's fused kernel.
 cudaError_t launch_render_bwd(int n, const RenderParams& p, const float* grad_out, float* grad_params, int num_sms,
                               int ctas_per_sm, cudaStream_t s);
 int render_bwd_max_ctas(int n);
@@ -85,6 +95,14 @@ cudaError_t noalloc_scratch(int device, unsigned char** out);
 cudaError_t render_noalloc(const RenderParams& proto, int64_t count, uint32_t want, unsigned char* base,
                            int num_sms, int* status, cudaStream_t s);
 
+// CTAs of a persistent kernel: `ctas` per SM, no more than there can be
+// galaxies.  (A CTA that finds the queue empty still starts up: 1672 CTAs for
+// 112 galaxies of 32 x 32 take longer than the galaxies.)
+inline int persistent_grid(const RenderParams& p, int ctas, int num_sms) {
+  const int64_t full = (int64_t)ctas * num_sms;
+  return (int)(full < p.max_galaxies ? full : p.max_galaxies > 0 ? p.max_galaxies : 1);
+}
+
 // Raises kernel `fn`'s dynamic shared-memory limit to `smem` bytes and
 // returns how many CTAs of `threads` threads fit on one SM, or -1 on
 // failure.  The limit belongs to the current device's context, so it is set
@@ -97,10 +115,6 @@ cudaError_t launch_render_fwd(int n, const RenderParams& p, int num_sms, int cta
 // profiles of p.records and p.records2 (N = 32, 64, 128; and 256).
 cudaError_t launch_render_fwd_composite(int n, const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s);
 cudaError_t launch_render_fwd256_composite(const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s);
-// Records of composites: the first profile's (batch p.b) at records, the
-// second's (batch `second`, same centre, size, PSF and patch) at records2.
-cudaError_t launch_composite_prep(const RenderParams& p, const BatchView& second, int64_t count,
-                                  unsigned char* records, unsigned char* records2, cudaStream_t s);
 cudaError_t launch_render_fwd256(const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s);
 // Resident CTAs per SM of the plain forward kernel for side n and radix
 // schedule `sched` (what the autotuner searches up to).

@@ -65,20 +65,20 @@ cudaError_t render_noalloc(const RenderParams& proto, int64_t count, uint32_t wa
   ps.small = reinterpret_cast<int32_t*>(base + OFF_SMALL);
   ps.order = reinterpret_cast<int32_t*>(base + OFF_ORDER);
   unsigned char* records = base + OFF_RECORDS;
-  // The array keeps the previous call's contents: the histogram must start
-  // at zero; everything else is rewritten before it is read.
-  cudaError_t e = cudaMemsetAsync(ps.hist, 0, KEYS * sizeof(int32_t), s);
-  if (e != cudaSuccess) return e;
-  e = launch_plan(proto.b, count, ps, FWD_BUCKETS, status, s);
-  if (e != cudaSuccess) return e;
   RenderParams p = proto;
+  p.max_galaxies = count;
   p.order = ps.order;
   p.bucket_start = ps.small;
   p.bucket_count = ps.small + NBUCKET;
   p.queue = ps.small + 2 * NBUCKET;
   p.records = records;
+  // The array keeps the previous call's contents: the histogram must start
+  // at zero; everything else is rewritten before it is read.
+  // (Small plans have no histogram.)
+  cudaError_t e = count > SMALL_PLAN ? cudaMemsetAsync(ps.hist, 0, KEYS * sizeof(int32_t), s) : cudaSuccess;
+  if (e != cudaSuccess) return e;
+  e = launch_plan_forward(p, count, ps, FWD_BUCKETS, records, s);
   p.chunk = 8;
-  e = launch_galaxy_prep(p, count, records, s);
   for (int b = 0; b < NBUCKET && e == cudaSuccess; ++b)
     if ((want >> b) & 1) e = launch_render_fwd(bucket_side(b), p, num_sms, 0, s);
   return e;

@@ -24,7 +24,6 @@
 //   reduce    warp shuffles, then one thread applies the chain rule
 #include "common.cuh"
 #include "internal.h"
-#include "lanczos_adj.cuh"
 
 namespace mog {
 
@@ -541,7 +540,7 @@ static cudaError_t launch_bwd_mode(const RenderParams& p, const float* grad_out,
   const int occ = bwd_occupancy<N, WN, EIG, LZ>();
   if (occ < 0) return cudaErrorInvalidConfiguration;
   const int ctas = (ctas_per_sm > 0 && ctas_per_sm < occ) ? ctas_per_sm : occ;
-  render_bwd_kernel<N, WN, EIG, LZ, CPG><<<ctas * num_sms, C::THREADS, C::SMEM, s>>>(p, grad_out, grad_params);
+  render_bwd_kernel<N, WN, EIG, LZ, CPG><<<persistent_grid(p, ctas, num_sms), C::THREADS, C::SMEM, s>>>(p, grad_out, grad_params);
   return cudaGetLastError();
 }
 
@@ -570,25 +569,6 @@ int render_bwd_max_ctas(int n) {
     case 256: return 1;
     default: return 0;
   }
-}
-
-// One warp per planned position (lane = mixture component).
-__global__ void adjoint_prep(RenderParams p, unsigned char* records) {
-  const int total = p.bucket_start[NBUCKET - 1] + p.bucket_count[NBUCKET - 1];
-  const int warps = (gridDim.x * blockDim.x) >> 5;
-  for (int pos = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; pos < total; pos += warps) {
-    const int64_t g = p.order[pos];
-    adjoint_record_warp(p.b, g, p.b.size[g], p.profiles, p.psfs, p.status, p.lanczos != 0,
-                        reinterpret_cast<AdjRecord*>(records + (size_t)pos * sizeof(AdjRecord)));
-    if (p.pcoef) eigen_coefficients_warp(p.b, g, p.psfs, p.pcoef, pos);
-    if (p.lanczos) lanczos_weights_and_slopes_warp(p.b, g, p.lzw + (size_t)pos * ADJ_LW);
-  }
-}
-
-cudaError_t launch_adjoint_prep(const RenderParams& p, int64_t count, unsigned char* records, cudaStream_t s) {
-  const int64_t blocks = (count + 7) / 8;
-  adjoint_prep<<<(int)(blocks < 8192 ? (blocks > 0 ? blocks : 1) : 8192), 256, 0, s>>>(p, records);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_render_bwd(int n, const RenderParams& p, const float* grad_out, float* grad_params, int num_sms,

@@ -412,7 +412,7 @@ cudaError_t launch_render_bwd256(const RenderParams& p, const float* grad_out, f
   const int occ = kernel_occupancy(reinterpret_cast<const void*>(fn), THREADS, smem);
   if (occ < 0) return cudaErrorInvalidConfiguration;
   // the scratch holds one slice per CTA, CTAS_PER_SM per SM
-  fn<<<num_sms * (occ < CTAS_PER_SM ? occ : CTAS_PER_SM), THREADS, smem, s>>>(p, grad_out, grad_params, scratch);
+  fn<<<persistent_grid(p, occ < CTAS_PER_SM ? occ : CTAS_PER_SM, num_sms), THREADS, smem, s>>>(p, grad_out, grad_params, scratch);
   return cudaGetLastError();
 }
 

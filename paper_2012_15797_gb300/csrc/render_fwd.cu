@@ -667,7 +667,7 @@ static cudaError_t launch_fwd_mode(const RenderParams& p, int num_sms, int ctas_
   const int occ = fwd_occupancy<N, LZ, EIG, V, LOSS, COMP>();
   if (occ < 0) return cudaErrorInvalidConfiguration;
   const int ctas = (ctas_per_sm > 0 && ctas_per_sm < occ) ? ctas_per_sm : occ;
-  render_fwd_kernel<N, LZ, EIG, CPG, V, LOSS, COMP><<<ctas * num_sms, C::THREADS, C::SMEM, s>>>(p);
+  render_fwd_kernel<N, LZ, EIG, CPG, V, LOSS, COMP><<<persistent_grid(p, ctas, num_sms), C::THREADS, C::SMEM, s>>>(p);
   return cudaGetLastError();
 }
 

@@ -514,7 +514,7 @@ static cudaError_t launch_fwd256(const RenderParams& p, int num_sms, int ctas_pe
   if (occ < 0) return cudaErrorInvalidConfiguration;
   // the accumulate mode's scratch holds one slice per CTA, CTAS_PER_SM per SM
   const int ctas = (ctas_per_sm > 0 && ctas_per_sm < occ) ? ctas_per_sm : occ;
-  render_fwd256_kernel<LZ, EIG, LOSS, COMP><<<num_sms * ctas, THREADS, Cfg256<COMP>::SMEM, s>>>(p);
+  render_fwd256_kernel<LZ, EIG, LOSS, COMP><<<persistent_grid(p, ctas, num_sms), THREADS, Cfg256<COMP>::SMEM, s>>>(p);
   return cudaGetLastError();
 }
 

@@ -283,7 +283,7 @@ cudaError_t launch_render_fwd64w(const RenderParams& p, int num_sms, int ctas_pe
   const int occ = render_fwd64w_max_ctas();
   if (occ < 0) return cudaErrorInvalidConfiguration;
   const int ctas = (ctas_per_sm > 0 && ctas_per_sm < occ) ? ctas_per_sm : occ;
-  render_fwd64w_kernel<<<ctas * num_sms, 32 * WARPS_PER_CTA, SMEM, s>>>(p);
+  render_fwd64w_kernel<<<persistent_grid(p, ctas, num_sms), 32 * WARPS_PER_CTA, SMEM, s>>>(p);
   return cudaGetLastError();
 }
 
