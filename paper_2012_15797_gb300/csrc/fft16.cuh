@@ -71,8 +71,14 @@ __device__ __forceinline__ void fft16_twiddles(int j, float2 (&tw)[15]) {
   for (int k1 = 1; k1 < 16; ++k1) sincospif(2.0f * (float)(j * k1) / (float)N, &tw[k1 - 1].y, &tw[k1 - 1].x);
 }
 
-template <int N, int S, class Write, class Read>
-__device__ __forceinline__ void fft16(const float2 (&tw)[15], float2 (&v)[16], Write write, Read read) {
+// `written` runs when the exchange's writes, which depend on every input of
+// the thread, have been issued.
+struct Nothing {
+  __device__ __forceinline__ void operator()() const {}
+};
+template <int N, int S, class Write, class Read, class Written = Nothing>
+__device__ __forceinline__ void fft16(const float2 (&tw)[15], float2 (&v)[16], Write write, Read read,
+                                      Written written = Written()) {
   constexpr int T = fft16_threads<N>();
   dft16<S>(v);
 #pragma unroll
@@ -81,6 +87,7 @@ __device__ __forceinline__ void fft16(const float2 (&tw)[15], float2 (&v)[16], W
     if (k1 > 0) x = (S > 0) ? cmul(x, tw[k1 - 1]) : cmulc(x, tw[k1 - 1]);
     *write(k1) = x;
   }
+  written();
   __syncwarp();
 #pragma unroll
   for (int q = 0; q < 16 / T; ++q)

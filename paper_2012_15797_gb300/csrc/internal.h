@@ -23,6 +23,7 @@ struct RenderParams {
   int* status;
   int chunk;                    // queue positions taken per request
   int64_t max_galaxies = INT64_MAX;   // upper bound of the bucket's galaxies (the batch's count): no more CTAs
+  int only_side = 0;            // 1: the batch names a single patch side (all its galaxies are in this bucket)
   int lanczos = 0;              // 1: sub-pixel shift by Lanczos convolution
   float* lzw = nullptr;         // lanczos: 16 floats per planned position, weights along x [0, 7), y [8, 15);
                                 // adjoint: ADJ_LW floats, weights and slopes
@@ -89,6 +90,11 @@ size_t render_bwd256_scratch_bytes(int num_sms);
 cudaError_t launch_render_bwd256(const RenderParams& p, const float* grad_out, float* grad_params, float2* scratch,
                                  int num_sms, cudaStream_t s);
 
+// The same adjoint (phase shift) with a cluster of CTAs per galaxy, for few
+// galaxies; needs no scratch.
+cudaError_t launch_render_bwd256_small(const RenderParams& p, const float* grad_out, float* grad_params, int num_sms,
+                                       cudaStream_t s);
+
 // Allocation-free forward render (noalloc.cu): the scratch of one call lives
 // in a fixed device array; noalloc_scratch returns its address on `device`.
 cudaError_t noalloc_scratch(int device, unsigned char** out);
@@ -125,6 +131,8 @@ cudaError_t launch_render_fwd64w(const RenderParams& p, int num_sms, int ctas_pe
 int render_fwd64w_max_ctas();
 size_t psf_spec64t_elems();
 cudaError_t launch_transpose_spec64(const float2* spec, float2* dst, cudaStream_t s);
+// The same renders with a cluster of CTAs per galaxy, for few galaxies.
+cudaError_t launch_render_fwd256_small(const RenderParams& p, int num_sms, cudaStream_t s);
 int render_fwd256_max_ctas(int sched);
 
 // Patch sides each direction supports (bit b: N = 32 << b).

@@ -244,6 +244,8 @@ __global__ void __launch_bounds__(256) plan_and_records(RenderParams p, BatchVie
   const int lane = threadIdx.x & 31;
   const int g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (g >= count) return;
+  // loss mode: NaN for the galaxies the kernels skip; the others overwrite theirs
+  if (KIND == Records::Forward && p.loss && lane == 0) p.chi2[g] = __int_as_float(0x7fffffff);
   const int key = plan_key(p.b, g, supported);
   if (key < 0) return;   // reported by the last CTA
   int before = 0;

@@ -404,6 +404,12 @@ size_t render_bwd256_scratch_bytes(int num_sms) {
 
 cudaError_t launch_render_bwd256(const RenderParams& p, const float* grad_out, float* grad_params, float2* scratch,
                                  int num_sms, cudaStream_t s) {
+  // Few galaxies: a cluster per galaxy (render_bwd256c.cu): 10 galaxies 92 -> 29
+  // us, 100 143 -> 81, about equal at 160 (a CTA of this kernel takes 90 to 140
+  // us for one, and a cluster has an SM per CTA).  The line is the batch's
+  // count; in a batch of several sides about one in twenty is 256 x 256.
+  if (!p.lanczos && p.max_galaxies <= (p.only_side ? 160 : 4096))
+    return launch_render_bwd256_small(p, grad_out, grad_params, num_sms, s);
   auto fn = p.lanczos ? (p.eigen ? (p.grad_n ? render_bwd256_kernel<true, true, true> : render_bwd256_kernel<false, true, true>)
                                  : (p.grad_n ? render_bwd256_kernel<true, false, true> : render_bwd256_kernel<false, false, true>))
                       : (p.eigen ? (p.grad_n ? render_bwd256_kernel<true, true, false> : render_bwd256_kernel<false, true, false>)

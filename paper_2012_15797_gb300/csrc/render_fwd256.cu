@@ -518,7 +518,21 @@ static cudaError_t launch_fwd256(const RenderParams& p, int num_sms, int ctas_pe
   return cudaGetLastError();
 }
 
+// Few galaxies: a cluster per galaxy (render_fwd256c.cu).  A CTA of this kernel
+// takes about 80 us for a galaxy, so below a few hundred galaxies the call takes
+// that long however few they are (10: 64 us on the earlier 512-thread CTAs, 30
+// on clusters; 400: 175 and 110), and up to a few thousand the last, partly
+// filled wave still weighs more than the clusters' lower rate (plain 0.206 us a
+// galaxy against 0.188, Lanczos 0.39 against 0.33).  The line is the batch's
+// count, the bucket's being known on the device only: with one side named it is
+// the bucket's, otherwise about one galaxy in twenty is 256 x 256.
+static bool few_galaxies(const RenderParams& p) {
+  const int64_t line = (p.lanczos || p.records2) ? 1500 : 3000;
+  return p.max_galaxies <= (p.only_side ? line : 16 * line);
+}
+
 cudaError_t launch_render_fwd256_composite(const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s) {
+  if (few_galaxies(p)) return launch_render_fwd256_small(p, num_sms, s);
   return p.lanczos ? launch_fwd256<true, false, false, true>(p, num_sms, ctas_per_sm, s)
                    : launch_fwd256<false, false, false, true>(p, num_sms, ctas_per_sm, s);
 }
@@ -526,6 +540,7 @@ cudaError_t launch_render_fwd256_composite(const RenderParams& p, int num_sms, i
 int render_fwd256_max_ctas(int) { return fwd256_occupancy<false, false, false, false>(); }
 
 cudaError_t launch_render_fwd256(const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s) {
+  if (few_galaxies(p)) return launch_render_fwd256_small(p, num_sms, s);
   if (p.loss)
     return p.eigen ? launch_fwd256<false, true, true>(p, num_sms, ctas_per_sm, s)
                    : launch_fwd256<false, false, true>(p, num_sms, ctas_per_sm, s);
