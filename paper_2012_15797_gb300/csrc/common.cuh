@@ -547,6 +547,26 @@ __device__ __forceinline__ float2 eigen_bin(const float2* spec, int elems, int k
   return acc;
 }
 
+// Bins at(0) .. at(M - 1) of it, component by component: M loads in flight per
+// thread, where a bin at a time waits for L2 k_eig times (renders with six
+// components: 10.6k galaxies of 256 x 256 8.10 -> 2.73 ms, 100k of 64 x 64
+// 1.94 -> 1.59, 124k of 32 x 32 0.81 -> 0.61; adjoints of 64 x 64 2.95 -> 2.53,
+// of 32 x 32 1.10 -> 0.93).
+template <int M, class At>
+__device__ __forceinline__ void eigen_bins(const float2* spec, int elems, int k_eig, const float* m, At at, float2 (&v)[M]) {
+#pragma unroll
+  for (int i = 0; i < M; ++i) v[i] = make_float2(0.0f, 0.0f);
+#pragma unroll 1
+  for (int c = 0; c < k_eig; ++c, spec += elems) {
+    float2 s[M];
+#pragma unroll
+    for (int i = 0; i < M; ++i) s[i] = __ldg(spec + at(i));
+    const float mc = m[c];
+#pragma unroll
+    for (int i = 0; i < M; ++i) v[i] = make_float2(fmaf(mc, s[i].x, v[i].x), fmaf(mc, s[i].y, v[i].y));
+  }
+}
+
 // One warp: the eigen-PSF terms of galaxy g at planned position `pos`.
 __device__ __forceinline__ void eigen_coefficients_warp(const BatchView& b, int64_t g, const DevPsf* psfs,
                                                         float* pcoef, int pos) {

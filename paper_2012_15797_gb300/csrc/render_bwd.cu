@@ -446,6 +446,11 @@ __global__ void __launch_bounds__(BwdCfg<N, CPG, WN, LZ>::THREADS, BwdCfg<N, CPG
             qp[k] = make_float2(qq[0], qq[1]);
           }
           adj_mixture_sums<BH / 2, WN>(s_fa, s_fc, s_fd, nf, qp, S, SQ, SN, SD);
+          [[maybe_unused]] float2 pe[BH];
+          if constexpr (EIG)
+            if (k_eig > 0)
+              eigen_bins(psf_hat + col * LS, C::PSF_ELEMS, k_eig, s_eigm,
+                         [&](int bb) { return stockham_out_index<N, R>(j, NS, (b0 + bb) / R, (b0 + bb) % R); }, pe);
 #pragma unroll
           for (int bb = 0; bb < BH; ++bb) {
             const int b = b0 + bb, q = b / R, m = b % R;
@@ -463,8 +468,7 @@ __global__ void __launch_bounds__(BwdCfg<N, CPG, WN, LZ>::THREADS, BwdCfg<N, CPG
             const float sq = (bb & 1) ? SQ[bb >> 1].y : SQ[bb >> 1].x;
             const float sn = (bb & 1) ? SN[bb >> 1].y : SN[bb >> 1].x;
             const float sd = (bb & 1) ? SD[bb >> 1].y : SD[bb >> 1].x;
-            const float2 pv = k_eig > 0 ? eigen_bin(psf_hat, C::PSF_ELEMS, k_eig, s_eigm, col * LS + l)
-                                        : __ldg(&psf_hat[col * LS + l]);
+            const float2 pv = (EIG && k_eig > 0) ? pe[bb] : __ldg(&psf_hat[col * LS + l]);
             float2 z;   // c_k conj(G) P phase
             if constexpr (LZ) {
               z = contract_shift(cscale(cmulc(pv, gk), ck), pxf, pxd, py[l], pyd[l], s, acc);

@@ -326,6 +326,11 @@ __global__ void __launch_bounds__(THREADS, LZ ? 1 : CTAS_PER_SM)
           qp[kk] = make_float2(qv[0], qv[1]);
         }
         adj_mixture_sums<2, WN>(s_fa, s_fc, s_fd, nf, qp, S, SQ, SN, SD);
+        [[maybe_unused]] float2 pe[4];
+        if constexpr (EIG)
+          if (k_eig > 0)
+            eigen_bins(psf_hat + k * LS, PSF_ELEMS, k_eig, s_eigm,
+                       [&](int bb) { return stockham_out_index<N, R2>(j, N / R2, (b0 + bb) / R2, (b0 + bb) % R2); }, pe);
 #pragma unroll
         for (int bb = 0; bb < 4; ++bb) {
           const int b = b0 + bb, qq = b / R2, m = b % R2;
@@ -342,7 +347,7 @@ __global__ void __launch_bounds__(THREADS, LZ ? 1 : CTAS_PER_SM)
           const float sq = (bb & 1) ? SQ[bb >> 1].y : SQ[bb >> 1].x;
           const float sn = (bb & 1) ? SN[bb >> 1].y : SN[bb >> 1].x;
           const float sd = (bb & 1) ? SD[bb >> 1].y : SD[bb >> 1].x;
-          const float2 pv = k_eig > 0 ? eigen_bin(psf_hat, PSF_ELEMS, k_eig, s_eigm, k * LS + l) : __ldg(&psf_hat[k * LS + l]);
+          const float2 pv = (EIG && k_eig > 0) ? pe[bb] : __ldg(&psf_hat[k * LS + l]);
           float2 z;
           if constexpr (LZ) {
             z = contract_shift(cscale(cmulc(pv, gk), ck), pxk, pxd[k], py[l], pyd[l], s, acc);

@@ -201,6 +201,10 @@ __global__ void __launch_bounds__(THREADS, 1)
           qp[i] = make_float2(fmaf(oa, fmaf(s22, oa, a1), a0), fmaf(ob, fmaf(s22, ob, a1), a0));
         }
         adj_mixture_sums<BH / 2, WN>(s_fa, s_fc, s_fd, nf, qp, S, SQ, SN, SD);
+        [[maybe_unused]] float2 pe[BH];
+        if constexpr (EIG)
+          if (k_eig > 0)
+            eigen_bins(psf_hat + k * LS + j, PSF_ELEMS, k_eig, pc, [&](int bb) { return 16 * (b0 + bb); }, pe);
 #pragma unroll
         for (int bb = 0; bb < BH; ++bb) {
           const int k2 = b0 + bb, l = j + 16 * k2;
@@ -216,7 +220,7 @@ __global__ void __launch_bounds__(THREADS, 1)
           const float sq = (bb & 1) ? SQ[bb >> 1].y : SQ[bb >> 1].x;
           const float sn = (bb & 1) ? SN[bb >> 1].y : SN[bb >> 1].x;
           const float sd = (bb & 1) ? SD[bb >> 1].y : SD[bb >> 1].x;
-          const float2 pv = k_eig > 0 ? eigen_bin(psf_hat, PSF_ELEMS, k_eig, pc, k * LS + l) : __ldg(&psf_hat[k * LS + l]);
+          const float2 pv = (EIG && k_eig > 0) ? pe[bb] : __ldg(&psf_hat[k * LS + l]);
           const float2 z = cscale(cmulc(cmul(pv, cmul(pxk, py[l])), gk), ck);   // c_k conj(G) P phase
           contract_bin(z, nu, om, s, sq, sn, acc);
           if constexpr (WN) acc[6] = fmaf(z.x, sd, acc[6]);

@@ -312,7 +312,14 @@ __global__ void __launch_bounds__(FwdCfg<N, CPG, V, COMP>::THREADS, FwdCfg<N, CP
     if (eig) {
       if constexpr (C::PSF_SMEM) {
         const DevPsf& ps = p.psfs[r.psf];
-        for (int e = tid; e < C::PSF_ELEMS; e += C::THREADS) psf_hat[e] = eigen_bin(ps.spec[B], C::PSF_ELEMS, ps.k_eig, pc, e);
+        constexpr int M = 5;   // bins per thread and pass
+        for (int e = tid; e < C::PSF_ELEMS; e += M * C::THREADS) {
+          float2 s[M];
+          eigen_bins(ps.spec[B], C::PSF_ELEMS, ps.k_eig, pc, [&](int i) { return min(e + i * C::THREADS, C::PSF_ELEMS - 1); }, s);
+#pragma unroll
+          for (int i = 0; i < M; ++i)
+            if (e + i * C::THREADS < C::PSF_ELEMS) psf_hat[e + i * C::THREADS] = s[i];
+        }
       }
       cur_psf = -1;   // the next galaxy forms its own
     } else if (need_psf) {   // uniform: every thread reads the same record

@@ -292,7 +292,9 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) render_fwd256c_kernel(Re
         // column nu = col / N; the second round from the far end of the block
         const int kl = cc ? KL - 1 - f : f, col = column(kl, rank);
         const float2* ph = psf_hat + col * LS + j;
-        if (!(EIG && k_eig)) {
+        if (EIG && k_eig) {
+          eigen_bins(ph, PSF_ELEMS, k_eig, pc, [](int m) { return m * T; }, v);
+        } else {
 #pragma unroll
           for (int m = 0; m < 16; ++m) v[m] = __ldg(ph + m * T);
         }
@@ -308,7 +310,6 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) render_fwd256c_kernel(Re
 #pragma unroll
         for (int m = 0; m < 16; ++m) {
           const int l = j + m * T;
-          if (EIG && k_eig) v[m] = eigen_bin(psf_hat, PSF_ELEMS, k_eig, pc, col * LS + l);
           const float2 ph = m < 8 ? cmul(pxk, py[l]) : cmulc(pxk, py[N - l]);
           v[m] = cscale(cmul(v[m], ph), (m & 1) ? s[m >> 1].y : s[m >> 1].x);
         }
