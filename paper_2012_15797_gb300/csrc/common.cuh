@@ -1078,16 +1078,19 @@ __device__ __forceinline__ void adj_component_tables(const AdjRecord& r, int c, 
   fd[c] = make_float4(r.fdq[c], r.fdq[c], r.fdn[c], r.fdn[c]);
 }
 
-// The Lanczos adjoint's bin: w = c_k conj(G) P, (px, pxd) the phase along nu
-// times the Lanczos response of the weights and of their slopes, (py, pyd)
-// along omega.  Adds d/dx and d/dy, the values through the slopes' responses,
-// and returns z = w px py for the other sums (contract_shape).
-__device__ __forceinline__ float2 contract_shift(float2 w, float2 px, float2 pxd, float2 py, float2 pyd, float s,
-                                                 float* acc) {
+// The Lanczos adjoint's bin, P = pv, G = gk: (px, pxd) the phase along nu times
+// the Lanczos response of the weights and of their slopes, (py, pyd) along
+// omega.  Adds d/dx and d/dy, the values through the slopes' responses, and
+// returns z = c_k conj(G) P px py for the other sums (contract_shape), formed as
+// in the plain adjoint: at integer offsets, where the responses are 1, those
+// sums are the same bit for bit.
+__device__ __forceinline__ float2 contract_shift(float2 pv, float2 gk, float ck, float2 px, float2 pxd, float2 py,
+                                                 float2 pyd, float s, float* acc) {
+  const float2 w = cscale(cmulc(pv, gk), ck);
   const float2 a = cmul(w, py), b = cmul(w, pyd);
   acc[1] = fmaf(fmaf(a.x, pxd.x, -a.y * pxd.y), s, acc[1]);
   acc[2] = fmaf(fmaf(b.x, px.x, -b.y * px.y), s, acc[2]);
-  return cmul(a, px);
+  return cscale(cmulc(cmul(pv, cmul(px, py)), gk), ck);
 }
 __device__ __forceinline__ void contract_shape(float zr, float nu, float om, float s, float sq, float sn, float* acc) {
   acc[0] = fmaf(zr, s, acc[0]);

@@ -471,7 +471,7 @@ __global__ void __launch_bounds__(BwdCfg<N, CPG, WN, LZ>::THREADS, BwdCfg<N, CPG
             const float2 pv = (EIG && k_eig > 0) ? pe[bb] : __ldg(&psf_hat[col * LS + l]);
             float2 z;   // c_k conj(G) P phase
             if constexpr (LZ) {
-              z = contract_shift(cscale(cmulc(pv, gk), ck), pxf, pxd, py[l], pyd[l], s, acc);
+              z = contract_shift(pv, gk, ck, pxf, pxd, py[l], pyd[l], s, acc);
               contract_shape(z.x, nu, om, s, sq, sn, acc);
             } else {
               const float2 bph = cmul(pv, cmul(pxf, py[l]));

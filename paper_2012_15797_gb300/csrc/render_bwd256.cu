@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(THREADS, LZ ? 1 : CTAS_PER_SM)
           const float2 pv = (EIG && k_eig > 0) ? pe[bb] : __ldg(&psf_hat[k * LS + l]);
           float2 z;
           if constexpr (LZ) {
-            z = contract_shift(cscale(cmulc(pv, gk), ck), pxk, pxd[k], py[l], pyd[l], s, acc);
+            z = contract_shift(pv, gk, ck, pxk, pxd[k], py[l], pyd[l], s, acc);
             contract_shape(z.x, nu, om, s, sq, sn, acc);
           } else {
             const float2 bph = cmul(pv, cmul(pxk, py[l]));
@@ -410,10 +410,13 @@ size_t render_bwd256_scratch_bytes(int num_sms) {
 cudaError_t launch_render_bwd256(const RenderParams& p, const float* grad_out, float* grad_params, float2* scratch,
                                  int num_sms, cudaStream_t s) {
   // Few galaxies: a cluster per galaxy (render_bwd256c.cu): 10 galaxies 92 -> 29
-  // us, 100 143 -> 81, about equal at 160 (a CTA of this kernel takes 90 to 140
-  // us for one, and a cluster has an SM per CTA).  The line is the batch's
-  // count; in a batch of several sides about one in twenty is 256 x 256.
-  if (!p.lanczos && p.max_galaxies <= (p.only_side ? 160 : 4096))
+  // us (Lanczos 106 -> 42), 100 143 -> 81 (118 -> 124), about equal at 160 (205
+  // -> 241): a CTA of this kernel takes 90 to 140 us for one, and a cluster has
+  // an SM per CTA.  The line is the batch's count; in a batch of several sides
+  // about one in twenty is 256 x 256 (1000 galaxies: Lanczos 177 -> 154 us, 4000:
+  // 413 -> 465).  One line for both shifts: at integer offsets they give the
+  // same gradients.
+  if (p.max_galaxies <= (p.only_side ? 128 : 2560))
     return launch_render_bwd256_small(p, grad_out, grad_params, num_sms, s);
   auto fn = p.lanczos ? (p.eigen ? (p.grad_n ? render_bwd256_kernel<true, true, true> : render_bwd256_kernel<false, true, true>)
                                  : (p.grad_n ? render_bwd256_kernel<true, false, true> : render_bwd256_kernel<false, false, true>))

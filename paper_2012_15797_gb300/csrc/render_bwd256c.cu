@@ -46,14 +46,21 @@ constexpr size_t off_py = off_w + sizeof(float2) * GROUPS * RS;
 constexpr size_t off_nb = off_py + sizeof(float2) * N;   // rank 0: nu = 1/2 column, P phase
 constexpr size_t off_ns = off_nb + sizeof(float2) * N;   // and the mixture sums
 constexpr size_t off_rec = (off_ns + sizeof(float) * 4 * N + 15) & ~size_t(15);
+// LZ: phase times slope response along omega; the nu = 1/2 column's P phase
+// with the slopes along x and along y; the phases times response and slope
+// response of the CTA's columns
+constexpr size_t LZ_ELEMS = 3 * N + 2 * KL;
 constexpr size_t off_terms = off_rec + 2 * sizeof(AdjRecord);
 constexpr size_t off_red = off_terms + sizeof(AdjTerms);
 constexpr size_t SMEM = off_red + sizeof(float) * 8 * CL * WARPS;
-static_assert(SMEM <= 227 * 1024, "shared memory of a CTA");
+constexpr size_t off_lz = SMEM;
+constexpr size_t SMEM_LZ = off_lz + sizeof(float2) * LZ_ELEMS;
+static_assert(SMEM_LZ <= 227 * 1024, "shared memory of a CTA");
 
 // WN: also d L / d(Sersic n), a seventh gradient per galaxy.  EIG: some PSF of
 // the context is an eigen-PSF (its spectrum combined bin by bin where read).
-template <bool WN, bool EIG>
+// LZ: the gradient of the Lanczos variant's model (see render_bwd.cu).
+template <bool WN, bool EIG, bool LZ>
 __global__ void __launch_bounds__(THREADS, 1)
     render_bwd256c_kernel(RenderParams p, const float* __restrict__ grad_out, float* __restrict__ grad_params) {
   constexpr float INV_N = 1.0f / N;
@@ -68,7 +75,13 @@ __global__ void __launch_bounds__(THREADS, 1)
   AdjRecord* rec = reinterpret_cast<AdjRecord*>(smem + off_rec);
   AdjTerms& at = *reinterpret_cast<AdjTerms*>(smem + off_terms);
   float* red = reinterpret_cast<float*>(smem + off_red);   // rank 0: [CTA][warp][8]
+  [[maybe_unused]] float2* pyd = reinterpret_cast<float2*>(smem + off_lz);
+  [[maybe_unused]] float2* nybx = pyd + N;   // rank 0
+  [[maybe_unused]] float2* nyby = pyd + 2 * N;
+  [[maybe_unused]] float2* px = pyd + 3 * N;
+  [[maybe_unused]] float2* pxd = px + KL;
   __shared__ float4 s_fa[KMAX], s_fc[KMAX], s_fd[KMAX];    // component tables of adj_mixture_sums
+  __shared__ float s_lw[LZ ? ADJ_LW : 1];                  // Lanczos weights and slopes
 
   const int tid = threadIdx.x;
   const int f = tid / T, j = tid % T;
@@ -104,15 +117,30 @@ __global__ void __launch_bounds__(THREADS, 1)
     const int nrt = r.nrc * ps.k, nr2 = real_terms_padded(nrt);
 
     // ---- per-galaxy tables; the nu = 1/2 column for the CTA of column 0 ----
-    const int t1 = N, t2 = t1 + (rank == 0 ? N : 0), t3 = t2 + nr2;
-    for (int i = tid; i < t3 + r.nf; i += THREADS) {
+    [[maybe_unused]] const float* lwg = LZ ? p.lzw + ((size_t)first + pos) * ADJ_LW : nullptr;
+    // a phase times the responses of the weights at `at` (and of their slopes, 8 on)
+    auto shift = [&](float2 ph, int at, float fr, float2& slope) {
+      float wv[7];
+      load_weights(lwg, at + 8, wv);
+      slope = cmul(ph, lanczos_response(wv, fr));
+      load_weights(lwg, at, wv);
+      return cmul(ph, lanczos_response(wv, fr));
+    };
+    const int t1 = N, t2 = t1 + (rank == 0 ? N : 0), t3 = t2 + nr2, t4 = t3 + r.nf;
+    for (int i = tid; i < t4 + (LZ ? KL : 0); i += THREADS) {
       if (i < t2) {
         const int l = i < t1 ? i : i - t1;
         const float om = (float)(l < N / 2 ? l : l - N) * INV_N;
         float2 phy;
+        [[maybe_unused]] float2 phyd;
         sincospif(-2.0f * r.y * om, &phy.y, &phy.x);
+        if constexpr (LZ) phy = shift(phy, 16, om, phyd);
         if (i < t1) {
           py[l] = phy;
+          if constexpr (LZ) {
+            pyd[l] = phyd;
+            if (l < ADJ_LW) s_lw[l] = lwg[l];
+          }
           continue;
         }
         const float q = fmaf(om, fmaf(r.s22, om, r.s12), 0.25f * r.s11);
@@ -125,10 +153,16 @@ __global__ void __launch_bounds__(THREADS, 1)
           if constexpr (WN) sd = fmaf(fmaf(r.fdq[c], q, r.fdn[c]), e, sd);
         }
         float2 phx;
+        [[maybe_unused]] float2 phxd;
         sincospif(-r.x, &phx.y, &phx.x);
+        if constexpr (LZ) phx = shift(phx, 0, 0.5f, phxd);
         const int e = (N / 2) * LS + l;
         const float2 pn = k_eig > 0 ? eigen_bin(psf_hat, PSF_ELEMS, k_eig, pc, e) : __ldg(psf_hat + e);
         nyb[l] = cmul(pn, cmul(phx, phy));
+        if constexpr (LZ) {
+          nybx[l] = cmul(pn, cmul(phxd, phy));
+          nyby[l] = cmul(pn, cmul(phx, phyd));
+        }
         nys[4 * l + 0] = s;
         nys[4 * l + 1] = sq;
         nys[4 * l + 2] = sn;
@@ -137,14 +171,20 @@ __global__ void __launch_bounds__(THREADS, 1)
         const int t = i - t2;
         if (t < nrt) adj_real_term(r, ps.mog, ps.k, N, t, &at, k_eig > 0 ? pc + 8 : nullptr);
         else adj_real_term_zero(t, &at);
-      } else {
+      } else if (!LZ || i < t4) {
         adj_component_tables(r, i - t3, s_fa, s_fc, s_fd);
+      } else if constexpr (LZ) {
+        const int kl = i - t4;
+        const float nu = (rank * KL + kl) * INV_N;
+        float2 ph;
+        sincospif(-2.0f * r.x * nu, &ph.y, &ph.x);
+        px[kl] = shift(ph, 0, nu, pxd[kl]);
       }
     }
     __syncthreads();
 
     float acc[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    adj_real_space<N, WN>(gpatch, N, at, nr2, rank * THREADS + tid, CL * THREADS, acc, r.s11, r.s12, r.s22);
+    adj_real_space<N, WN, LZ>(gpatch, N, at, nr2, rank * THREADS + tid, CL * THREADS, acc, r.s11, r.s12, r.s22, s_lw);
 
     // ---- rows ----
     float2 v[16];
@@ -188,7 +228,9 @@ __global__ void __launch_bounds__(THREADS, 1)
       const float a0 = s11 * nu * nu, a1 = s12x2 * nu;
       const int nf = r.nf;
       float2 pxk;
-      sincospif(-2.0f * r.x * nu, &pxk.y, &pxk.x);
+      [[maybe_unused]] const float2 pxdk = LZ ? pxd[cc * GROUPS + f] : make_float2(0.f, 0.f);
+      if constexpr (LZ) pxk = px[cc * GROUPS + f];
+      else sincospif(-2.0f * r.x * nu, &pxk.y, &pxk.x);
       constexpr int BH = 8;   // bins per sweep over the components
 #pragma unroll
       for (int b0 = 0; b0 < 16; b0 += BH) {
@@ -221,12 +263,24 @@ __global__ void __launch_bounds__(THREADS, 1)
           const float sn = (bb & 1) ? SN[bb >> 1].y : SN[bb >> 1].x;
           const float sd = (bb & 1) ? SD[bb >> 1].y : SD[bb >> 1].x;
           const float2 pv = (EIG && k_eig > 0) ? pe[bb] : __ldg(&psf_hat[k * LS + l]);
-          const float2 z = cscale(cmulc(cmul(pv, cmul(pxk, py[l])), gk), ck);   // c_k conj(G) P phase
-          contract_bin(z, nu, om, s, sq, sn, acc);
+          float2 z;   // c_k conj(G) P phase
+          if constexpr (LZ) {
+            z = contract_shift(pv, gk, ck, pxk, pxdk, py[l], pyd[l], s, acc);
+            contract_shape(z.x, nu, om, s, sq, sn, acc);
+          } else {
+            z = cscale(cmulc(cmul(pv, cmul(pxk, py[l])), gk), ck);
+            contract_bin(z, nu, om, s, sq, sn, acc);
+          }
           if constexpr (WN) acc[6] = fmaf(z.x, sd, acc[6]);
           if (k == 0) {
             const float2 zh = cmulc(nyb[l], gn);
-            contract_bin(zh, 0.5f, om, nys[4 * l], nys[4 * l + 1], nys[4 * l + 2], acc);
+            if constexpr (LZ) {
+              acc[1] = fmaf(fmaf(nybx[l].x, gn.x, nybx[l].y * gn.y), nys[4 * l], acc[1]);
+              acc[2] = fmaf(fmaf(nyby[l].x, gn.x, nyby[l].y * gn.y), nys[4 * l], acc[2]);
+              contract_shape(zh.x, 0.5f, om, nys[4 * l], nys[4 * l + 1], nys[4 * l + 2], acc);
+            } else {
+              contract_bin(zh, 0.5f, om, nys[4 * l], nys[4 * l + 1], nys[4 * l + 2], acc);
+            }
             if constexpr (WN) acc[6] = fmaf(zh.x, nys[4 * l + 3], acc[6]);
           }
         }
@@ -251,8 +305,8 @@ __global__ void __launch_bounds__(THREADS, 1)
       float* out = grad_params + r.gal * NACC;
       if constexpr (WN) out[6] = t[6];
       out[0] = t[0] / r.flux;
-      out[1] = TWO_PI * t[1];
-      out[2] = TWO_PI * t[2];
+      out[1] = (LZ ? 1.0f : TWO_PI) * t[1];
+      out[2] = (LZ ? 1.0f : TWO_PI) * t[2];
 #pragma unroll
       for (int c = 0; c < 3; ++c) out[3 + c] = t[3] * r.dS[c][0] + t[4] * r.dS[c][1] + t[5] * r.dS[c][2];
     }
@@ -263,13 +317,16 @@ __global__ void __launch_bounds__(THREADS, 1)
 
 cudaError_t launch_render_bwd256_small(const RenderParams& p, const float* grad_out, float* grad_params, int num_sms,
                                        cudaStream_t s) {
-  auto fn = p.eigen ? (p.grad_n ? render_bwd256c_kernel<true, true> : render_bwd256c_kernel<false, true>)
-                    : (p.grad_n ? render_bwd256c_kernel<true, false> : render_bwd256c_kernel<false, false>);
-  if (kernel_occupancy(reinterpret_cast<const void*>(fn), THREADS, SMEM) < 0) return cudaErrorInvalidConfiguration;
+  auto fn = p.lanczos ? (p.eigen ? (p.grad_n ? render_bwd256c_kernel<true, true, true> : render_bwd256c_kernel<false, true, true>)
+                                 : (p.grad_n ? render_bwd256c_kernel<true, false, true> : render_bwd256c_kernel<false, false, true>))
+                      : (p.eigen ? (p.grad_n ? render_bwd256c_kernel<true, true, false> : render_bwd256c_kernel<false, true, false>)
+                                 : (p.grad_n ? render_bwd256c_kernel<true, false, false> : render_bwd256c_kernel<false, false, false>));
+  const size_t smem = p.lanczos ? SMEM_LZ : SMEM;
+  if (kernel_occupancy(reinterpret_cast<const void*>(fn), THREADS, smem) < 0) return cudaErrorInvalidConfiguration;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(persistent_grid(p, 1, num_sms / CL) * CL));
   cfg.blockDim = dim3(THREADS);
-  cfg.dynamicSmemBytes = SMEM;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;

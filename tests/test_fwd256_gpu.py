@@ -3,7 +3,9 @@ a galaxy that is skipped in the middle.  Forward, every mode: batch sizes
 around the pipeline depth of the cluster kernel that small batches take (tables
 one galaxy ahead, records three ahead), and one above the line from which a CTA
 renders a galaxy: max |d pixel| <= 2e-6 flux (the render tolerance).  Adjoint:
-both kernels agree with the oracle's gradients within the adjoint tolerance."""
+both kernels agree with the oracle's gradients within the adjoint tolerance;
+at integer offsets the Lanczos shift does the same operations as the phase
+shift, so that every gradient but x and y is the same."""
 
 import numpy as np
 import pytest
@@ -105,3 +107,25 @@ def test_adjoint_parity_with_skipped_galaxies(gpu_renderer, tables, sersic, coun
         if sersic:
             dn = float(np.sum(A.sersic_derivative(g, hat, psf.mog, tables) * pix))
             assert abs(got[i, 6] - dn) <= 1e-4 * abs(dn) + 1e-5 * norm * abs(g["flux"]), i
+
+
+@pytest.mark.parametrize("count", [1, 41, 300])
+def test_lanczos_adjoint_small_and_large_batches(gpu_renderer, tables, count):
+    import torch
+    from paper_2012_15797_gb300.renderer import to_device
+    from test_lanczos_adjoint_gpu import check, oracle_grads_lanczos
+    gals = _batch(count, None)
+    b = to_device(gals)
+    go = torch.randn(b.total, generator=torch.Generator(device="cuda").manual_seed(count), device="cuda")
+    got = gpu_renderer.render_backward(b, go, shift="lanczos")
+    last = [go[int(b.offsets[-1]):].double().cpu().numpy().reshape(256, 256)]
+    one = gals.subset(np.array([count - 1]))
+    check(got[-1:].double().cpu().numpy(), oracle_grads_lanczos(one, gpu_renderer.psfs, tables, last), one, last)
+    gals.x[:] = np.round(gals.x * 4)
+    gals.y[:] = np.round(gals.y * 4)
+    b = to_device(gals)
+    lz = gpu_renderer.render_backward(b, go, shift="lanczos")
+    phase = gpu_renderer.render_backward(b, go)
+    gpu_renderer.sync_status()
+    cols = [0, 3, 4, 5]
+    assert torch.equal(lz[:, cols], phase[:, cols])
