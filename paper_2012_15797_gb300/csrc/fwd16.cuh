@@ -78,4 +78,75 @@ __device__ __forceinline__ void mixture16(const float4* fc, int nf, float s11, f
   }
 }
 
+// Real-space part of a Lanczos-shifted galaxy: Lz(R), R the nr terms at the
+// integer offset, Lz the periodic Lanczos convolution with weights wl (x:
+// [0, 7), y: [8, 15)), in strips of STRIP rows: the rows a strip needs are
+// evaluated and convolved along x (8 pixels of two rows per thread, neighbours
+// by shuffle) into `strip`, shared memory of (STRIP + 6) rows, then along y;
+// add(y, x0, acc) takes 8 pixels of the result.  Called by all threads; starts
+// writing `strip` at once and ends with a CTA barrier.
+template <int N, int STRIP, int THREADS, int R, class Add>
+__device__ __forceinline__ void lanczos_real_strips(const RealTermsN<R>& rt, int nr, const float* wl, float* strip, Add add) {
+  static_assert(STRIP % 2 == 0 && N % STRIP == 0, "rows in pairs, whole strips");
+  constexpr int LANES = N / 8, GROUPS = THREADS / LANES;   // lanes per row
+  const int j = threadIdx.x % LANES, g = threadIdx.x / LANES;
+  const unsigned lanes = (0xffffffffu >> (32 - LANES)) << (threadIdx.x & 31 & ~(LANES - 1));
+  const int x0 = 8 * j;
+  float wx[7], wy[7];
+#pragma unroll
+  for (int a = 0; a < 7; ++a) {
+    wx[a] = wl[a];
+    wy[a] = wl[8 + a];
+  }
+#pragma unroll 1
+  for (int y0 = 0; y0 < N; y0 += STRIP) {
+    // rows y0 - 3 .. y0 + STRIP + 2 (mod N), two at a time, convolved along x
+    for (int i = 2 * g; i < STRIP + 6; i += 2 * GROUPS) {
+      float2 r[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) r[u] = make_float2(0.0f, 0.0f);
+      real_space_rows(rt, nr, (float)((y0 - 3 + i) & (N - 1)), (float)((y0 - 2 + i) & (N - 1)), (float)x0, r);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float win[14];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) win[3 + u] = h ? r[u].y : r[u].x;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {   // x0 - 3 + a from the lane below, x0 + 8 + a from the lane above
+          win[a] = __shfl_sync(lanes, h ? r[5 + a].y : r[5 + a].x, (j + LANES - 1) % LANES, LANES);
+          win[11 + a] = __shfl_sync(lanes, h ? r[a].y : r[a].x, (j + 1) % LANES, LANES);
+        }
+        float X[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          float acc = 0.0f;
+#pragma unroll
+          for (int a = 0; a < 7; ++a) acc = fmaf(wx[a], win[3 + u - (a - 3)], acc);
+          X[u] = acc;
+        }
+        float4* srow = reinterpret_cast<float4*>(strip + (i + h) * N + x0);
+        srow[0] = make_float4(X[0], X[1], X[2], X[3]);
+        srow[1] = make_float4(X[4], X[5], X[6], X[7]);
+      }
+    }
+    __syncthreads();
+    // output rows y0 + o: sum_b wy_b X(y - b), strip rows o + 3 - b
+    for (int o = g; o < STRIP; o += GROUPS) {
+      float acc[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) acc[u] = 0.0f;
+#pragma unroll
+      for (int b = 0; b < 7; ++b) {
+        const float4* srow = reinterpret_cast<const float4*>(strip + (o + 6 - b) * N + x0);
+        const float4 p0 = srow[0], p1 = srow[1];
+        const float v[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc[u] = fmaf(wy[b], v[u], acc[u]);
+      }
+      add(y0 + o, x0, acc);
+    }
+    __syncthreads();
+  }
+}
+
 }  // namespace mog

@@ -116,6 +116,10 @@ inline int persistent_grid(const RenderParams& p, int ctas, int num_sms) {
 // device configures it there.
 int kernel_occupancy(const void* fn, int threads, size_t smem);
 
+// 128 x 128, 16 values per thread (render_fwd128.cu): every variant of the first
+// schedule (composites when p.records2 is set).
+cudaError_t launch_render_fwd128(const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s);
+int render_fwd128_max_ctas();
 cudaError_t launch_render_fwd(int n, const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s);
 // Composites (mog_render_composite): one transform per galaxy for the two
 // profiles of p.records and p.records2 (N = 32, 64, 128; and 256).
@@ -139,7 +143,6 @@ int render_fwd256_max_ctas(int sched);
 constexpr uint32_t FWD_BUCKETS = 0xF;   // 32, 64, 128, 256
 constexpr uint32_t LZ_BUCKETS = 0xF;    // Lanczos variant: 32, 64, 128, 256
 constexpr uint32_t BWD_BUCKETS = 0xF;   // 32, 64, 128, 256
-size_t render_fwd_smem(int n);
 
 // Gaussian-mixture fits of `count` h x w PSF images (psf_fit.cu).
 cudaError_t launch_psf_fit(const float* images, int count, int h, int w, int k, int iters, float* rows,

@@ -650,18 +650,15 @@ __global__ void __launch_bounds__(FwdCfg<N, CPG, V, COMP>::THREADS, FwdCfg<N, CP
 }
 
 // Columns per group of the launched kernel: two at N = 128 (two 512-thread
-// CTAs per SM), except in the Lanczos variant.
-template <int N, bool LZ>
-constexpr int fwd_cpg() { return (N == 128 && !LZ) ? 2 : 1; }
+// CTAs per SM).
+template <int N>
+constexpr int fwd_cpg() { return N == 128 ? 2 : 1; }
 
-static_assert(2 * (FwdCfg<128, 2>::SMEM + 1024) <= 228 * 1024, "two 128 x 128 CTAs share an SM's shared memory");
-
-static_assert(2 * (FwdCfg<128, 2, 0, true>::SMEM + 1024) <= 228 * 1024, "two 128 x 128 composite CTAs share an SM");
-static_assert(FwdCfg<128, 1, 0, true>::SMEM <= 227 * 1024, "the Lanczos composite CTA fits an SM's shared memory");
+static_assert(2 * (FwdCfg<128, 2, 1>::SMEM + 1024) <= 228 * 1024, "two 128 x 128 CTAs share an SM's shared memory");
 
 template <int N, bool LZ = false, bool EIG = false, int V = 0, bool LOSS = false, bool COMP = false>
 static int fwd_occupancy() {
-  constexpr int CPG = fwd_cpg<N, LZ>();
+  constexpr int CPG = fwd_cpg<N>();
   using C = FwdCfg<N, CPG, V, COMP>;
   return kernel_occupancy(reinterpret_cast<const void*>(render_fwd_kernel<N, LZ, EIG, CPG, V, LOSS, COMP>),
                           C::THREADS, C::SMEM);
@@ -669,7 +666,7 @@ static int fwd_occupancy() {
 
 template <int N, bool LZ, bool EIG, int V, bool LOSS = false, bool COMP = false>
 static cudaError_t launch_fwd_mode(const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s) {
-  constexpr int CPG = fwd_cpg<N, LZ>();
+  constexpr int CPG = fwd_cpg<N>();
   using C = FwdCfg<N, CPG, V, COMP>;
   const int occ = fwd_occupancy<N, LZ, EIG, V, LOSS, COMP>();
   if (occ < 0) return cudaErrorInvalidConfiguration;
@@ -690,10 +687,15 @@ static cudaError_t launch_fwd(const RenderParams& p, int num_sms, int ctas_per_s
                      : launch_fwd_mode<N, false, true, 0>(p, num_sms, ctas_per_sm, s);
   if (p.lanczos) return launch_fwd_mode<N, true, false, 0>(p, num_sms, ctas_per_sm, s);
   if (N == 64 && p.sched == 2) return launch_render_fwd64w(p, num_sms, ctas_per_sm, s);
-  if constexpr (N == 128)
-    if (p.sched == 2) return launch_fwd_mode<N, false, false, 2>(p, num_sms, ctas_per_sm, s);
   return p.sched == 1 ? launch_fwd_mode<N, false, false, 1>(p, num_sms, ctas_per_sm, s)
                       : launch_fwd_mode<N, false, false, 0>(p, num_sms, ctas_per_sm, s);
+}
+
+// 128 x 128: the first schedule is render_fwd128.cu's.
+static cudaError_t launch_fwd_128(const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s) {
+  if (p.sched == 0 || p.loss || p.eigen || p.lanczos) return launch_render_fwd128(p, num_sms, ctas_per_sm, s);
+  return p.sched == 2 ? launch_fwd_mode<128, false, false, 2>(p, num_sms, ctas_per_sm, s)
+                      : launch_fwd_mode<128, false, false, 1>(p, num_sms, ctas_per_sm, s);
 }
 
 template <int N>
@@ -706,7 +708,7 @@ cudaError_t launch_render_fwd_composite(int n, const RenderParams& p, int num_sm
   switch (n) {
     case 32: return launch_fwd_composite<32>(p, num_sms, ctas_per_sm, s);
     case 64: return launch_fwd_composite<64>(p, num_sms, ctas_per_sm, s);
-    case 128: return launch_fwd_composite<128>(p, num_sms, ctas_per_sm, s);
+    case 128: return launch_render_fwd128(p, num_sms, ctas_per_sm, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -715,7 +717,7 @@ cudaError_t launch_render_fwd(int n, const RenderParams& p, int num_sms, int cta
   switch (n) {
     case 32: return launch_fwd<32>(p, num_sms, ctas_per_sm, s);
     case 64: return launch_fwd<64>(p, num_sms, ctas_per_sm, s);
-    case 128: return launch_fwd<128>(p, num_sms, ctas_per_sm, s);
+    case 128: return launch_fwd_128(p, num_sms, ctas_per_sm, s);
     case 256: return launch_render_fwd256(p, num_sms, ctas_per_sm, s);
     default: return cudaErrorInvalidValue;
   }
@@ -727,17 +729,8 @@ int render_fwd_max_ctas(int n, int sched) {
     case 64: return sched == 2 ? render_fwd64w_max_ctas()
                   : sched == 1 ? fwd_occupancy<64, false, false, 1>() : fwd_occupancy<64>();
     case 128: return sched == 2   ? fwd_occupancy<128, false, false, 2>()
-                     : sched == 1 ? fwd_occupancy<128, false, false, 1>() : fwd_occupancy<128>();
+                     : sched == 1 ? fwd_occupancy<128, false, false, 1>() : render_fwd128_max_ctas();
     case 256: return render_fwd256_max_ctas(sched);
-    default: return 0;
-  }
-}
-
-size_t render_fwd_smem(int n) {
-  switch (n) {
-    case 32: return FwdCfg<32>::SMEM;
-    case 64: return FwdCfg<64>::SMEM;
-    case 128: return FwdCfg<128, fwd_cpg<128, false>()>::SMEM;
     default: return 0;
   }
 }

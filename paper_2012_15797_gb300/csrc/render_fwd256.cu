@@ -83,78 +83,10 @@ struct Cfg256 {
   static_assert(CTAS_PER_SM * (SMEM + 512 + 1024) <= 228 * 1024, "two CTAs share an SM's shared memory");
 };
 
-// LZ, galaxy with real-space terms: patch += Lz(R), R the real-space terms at
-// the integer offset, Lz the periodic Lanczos convolution with weights wl
-// (x: [0, 7), y: [8, 15)).  Called by all threads after the patch holds the
-// Fourier part; `strip` is shared memory of (STRIP + 6) rows.
-template <int RC>
-__device__ __forceinline__ void lanczos_real_256(const RealTermsN<RC>& rt, int nr, const float* wl, float* strip,
-                                                 float* dst) {
-  const int j = threadIdx.x & 31;
-  const int x0 = 8 * j;
-  float wx[7], wy[7];
-#pragma unroll
-  for (int a = 0; a < 7; ++a) {
-    wx[a] = wl[a];
-    wy[a] = wl[8 + a];
-  }
-  for (int y0 = 0; y0 < N; y0 += STRIP) {
-    // rows y0 - 3 .. y0 + STRIP + 2 (mod N), two at a time, convolved along x
-    for (int i = 2 * (threadIdx.x >> 5); i < STRIP + 6; i += 2 * WARPS) {
-      float2 R[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) R[u] = make_float2(0.0f, 0.0f);
-      real_space_rows(rt, nr, (float)((y0 - 3 + i) & (N - 1)), (float)((y0 - 2 + i) & (N - 1)), (float)x0, R);
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        float win[14];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) win[3 + u] = h ? R[u].y : R[u].x;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {   // x0 - 3 + a from the lane below, x0 + 8 + a from the lane above
-          win[a] = __shfl_sync(0xffffffffu, h ? R[5 + a].y : R[5 + a].x, (j + 31) & 31);
-          win[11 + a] = __shfl_sync(0xffffffffu, h ? R[a].y : R[a].x, (j + 1) & 31);
-        }
-        float X[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          float acc = 0.0f;
-#pragma unroll
-          for (int a = 0; a < 7; ++a) acc = fmaf(wx[a], win[3 + u - (a - 3)], acc);
-          X[u] = acc;
-        }
-        float4* srow = reinterpret_cast<float4*>(strip + (i + h) * N + x0);
-        srow[0] = make_float4(X[0], X[1], X[2], X[3]);
-        srow[1] = make_float4(X[4], X[5], X[6], X[7]);
-      }
-    }
-    __syncthreads();
-    // output rows y0 + o: sum_b wy_b X(y - b), strip rows o + 3 - b
-    for (int o = threadIdx.x >> 5; o < STRIP; o += WARPS) {
-      float acc[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) acc[u] = 0.0f;
-#pragma unroll
-      for (int b = 0; b < 7; ++b) {
-        const float4* srow = reinterpret_cast<const float4*>(strip + (o + 6 - b) * N + x0);
-        const float4 p0 = srow[0], p1 = srow[1];
-        const float v[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
-#pragma unroll
-        for (int u = 0; u < 8; ++u) acc[u] = fmaf(wy[b], v[u], acc[u]);
-      }
-      float4* d = reinterpret_cast<float4*>(dst + (y0 + o) * N + x0);
-      const float4 f0 = d[0], f1 = d[1];   // the Fourier part, written by this CTA
-      d[0] = make_float4(f0.x + acc[0], f0.y + acc[1], f0.z + acc[2], f0.w + acc[3]);
-      d[1] = make_float4(f1.x + acc[4], f1.y + acc[5], f1.z + acc[6], f1.w + acc[7]);
-    }
-    __syncthreads();
-  }
-}
-
 // LZ: the Lanczos sub-pixel shift (records carry the integer offset and the
 // fraction): the convolution of the Fourier part is folded into the phase
-// tables, the real-space part is convolved along x, // then along y, in strips.  EIG: some PSF of the context is an eigen-PSF.
-// LOSS: the loss mode of mog_render_chi2.  COMP: composites of two profiles
+// tables, the real-space part is convolved along x, then along y, in strips.
+// EIG: some PSF of the context is an eigen-PSF.  LOSS: the loss mode of mog_render_chi2.  COMP: composites of two profiles
 // (p.records2).
 template <bool LZ, bool EIG, bool LOSS, bool COMP>
 __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) render_fwd256_kernel(RenderParams p) {
@@ -486,7 +418,14 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) render_fwd256_kernel(Ren
     if constexpr (LZ) {
       if (nrt > 0) {   // uniform
         __syncthreads();   // the whole Fourier part is in the patch; W is free
-        lanczos_real_256(rt, nrt, s_lzw[LZ ? buf : 0], reinterpret_cast<float*>(smem), p.out + off);
+        float* const dst = p.out + off;
+        lanczos_real_strips<N, STRIP, THREADS>(
+            rt, nrt, s_lzw[LZ ? buf : 0], reinterpret_cast<float*>(smem), [&](int y, int x0, const float(&acc)[8]) {
+              float4* const d = reinterpret_cast<float4*>(dst + y * N + x0);
+              const float4 f0 = d[0], f1 = d[1];   // the Fourier part, written by this CTA
+              d[0] = make_float4(f0.x + acc[0], f0.y + acc[1], f0.z + acc[2], f0.w + acc[3]);
+              d[1] = make_float4(f1.x + acc[4], f1.y + acc[5], f1.z + acc[6], f1.w + acc[7]);
+            });
       }
     }
     pos = pos1;

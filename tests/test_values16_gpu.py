@@ -1,11 +1,12 @@
-"""The 256 x 256 kernels with 16 values per thread against the FP64 oracle, with
-a galaxy that is skipped in the middle.  Forward, every mode: batch sizes
-around the pipeline depth of the cluster kernel that small batches take (tables
-one galaxy ahead, records three ahead), and one above the line from which a CTA
-renders a galaxy: max |d pixel| <= 2e-6 flux (the render tolerance).  Adjoint:
-both kernels agree with the oracle's gradients within the adjoint tolerance;
-at integer offsets the Lanczos shift does the same operations as the phase
-shift, so that every gradient but x and y is the same."""
+"""The kernels with 16 values per thread (256 x 256, 128 x 128) against the FP64
+oracle, with a galaxy that is skipped in the middle.  Forward, every mode: batch
+sizes around the pipeline depth (tables one galaxy ahead, records three ahead),
+for 256 x 256 below and above the line from which a CTA and no longer a cluster
+renders a galaxy: max |d pixel| <= 2e-6 flux (the render tolerance); adding to
+an image gives the image plus the model.  Adjoint: every kernel agrees with the
+oracle's gradients within the adjoint tolerance; at integer offsets the Lanczos
+shift does the same operations as the phase shift, so that every gradient but x
+and y is the same."""
 
 import numpy as np
 import pytest
@@ -19,8 +20,8 @@ pytestmark = pytest.mark.gpu
 TOL = 2e-6
 
 
-def _batch(count, bad):
-    rows = [_row(**{"size": 256, "x": 0.37 - 0.1 * (i % 7), "y": -0.21 + 0.05 * (i % 7), **EDGE[(i % 7) % len(EDGE)]})
+def _batch(count, bad, size=256):
+    rows = [_row(**{"size": size, "x": 0.37 - 0.1 * (i % 7), "y": -0.21 + 0.05 * (i % 7), **EDGE[(i % 7) % len(EDGE)]})
             for i in range(count)]
     gals = _gals(rows)
     if bad is not None:
@@ -29,14 +30,15 @@ def _batch(count, bad):
 
 
 @pytest.mark.parametrize("mode", ["phase", "lanczos", "loss", "composite"])
-@pytest.mark.parametrize("count,bad", [(1, None), (2, 0), (3, 1), (7, 3), (640, 637)])
-def test_parity_with_skipped_galaxies(gpu_renderer, tables, mode, count, bad):
+@pytest.mark.parametrize("size,count,bad", [(256, 1, None), (256, 2, 0), (256, 3, 1), (256, 7, 3), (256, 640, 637),
+                                            (128, 1, None), (128, 2, 0), (128, 3, 1), (128, 640, 637)])
+def test_parity_with_skipped_galaxies(gpu_renderer, tables, mode, size, count, bad):
     import torch
     from paper_2012_15797_gb300 import capi
     from paper_2012_15797_gb300.renderer import patches, to_device
-    gals = _batch(count, bad)
+    gals = _batch(count, bad, size)
     # one CTA per SM and long queue chunks: a CTA takes several galaxies in turn
-    capi.mog_set_launch_shape(gpu_renderer.ctx, 0, 256, 1, 8, 0)
+    capi.mog_set_launch_shape(gpu_renderer.ctx, 0, size, 1, 8, 0)
     try:
         b = to_device(gals)
         out = torch.full((b.total,), 7.0, device="cuda")
@@ -55,7 +57,7 @@ def test_parity_with_skipped_galaxies(gpu_renderer, tables, mode, count, bad):
             with pytest.raises(capi.MogError):
                 gpu_renderer.sync_status()
     finally:
-        capi.mog_set_launch_shape(gpu_renderer.ctx, 0, 256, 0, 1, 0)
+        capi.mog_set_launch_shape(gpu_renderer.ctx, 0, size, 0, 1, 0)
     got = patches(out, b)
     for i in range(max(0, count - 7), count):
         if i == bad:
@@ -129,3 +131,16 @@ def test_lanczos_adjoint_small_and_large_batches(gpu_renderer, tables, count):
     gpu_renderer.sync_status()
     cols = [0, 3, 4, 5]
     assert torch.equal(lz[:, cols], phase[:, cols])
+
+
+@pytest.mark.parametrize("mode", ["phase", "lanczos"])
+@pytest.mark.parametrize("size", [128, 256])
+def test_adding_to_an_image_is_the_image_plus_the_model(gpu_renderer, mode, size):
+    import torch
+    from paper_2012_15797_gb300.renderer import to_device
+    b = to_device(_batch(9, None, size))
+    base = torch.randn(b.total, device="cuda")
+    out = base.clone()
+    gpu_renderer.render(b, out, shift=mode, add=True)
+    assert torch.equal(out, base + gpu_renderer.render(b, shift=mode))
+    gpu_renderer.sync_status()
