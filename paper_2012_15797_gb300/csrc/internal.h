@@ -84,6 +84,10 @@ cudaError_t launch_plan_composite(const RenderParams& p, const BatchView& second
 cudaError_t launch_render_bwd(int n, const RenderParams& p, const float* grad_out, float* grad_params, int num_sms,
                               int ctas_per_sm, cudaStream_t s);
 int render_bwd_max_ctas(int n);
+// 128 x 128 adjoint, 16 values per thread (render_bwd128.cu).
+cudaError_t launch_render_bwd128(const RenderParams& p, const float* grad_out, float* grad_params, int num_sms,
+                                 int ctas_per_sm, cudaStream_t s);
+int render_bwd128_max_ctas();
 // 256 x 256 adjoint (and forward render adding to its patches): need
 // render_bwd256_scratch_bytes(num_sms) of global scratch, one slice per CTA.
 size_t render_bwd256_scratch_bytes(int num_sms);

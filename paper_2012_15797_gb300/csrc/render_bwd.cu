@@ -27,24 +27,17 @@
 
 namespace mog {
 
-// CPG: row pairs (and columns) each group of TPF threads transforms, one
-// after the other.  CPG = 2 (N = 128) halves the CTA to 512 threads and its
-// shared memory (the gradient rows are read from global memory, L2-resident,
-// instead of being staged, and the row transforms use one work row per
-// group), so two CTAs share an SM and one computes while the other waits at a
-// CTA barrier.
+// Sides 32 and 64 (128 and 256: render_bwd128.cu, render_bwd256.cu).
 // WN: the variant with the Sersic-index gradient (one more mixture sum per
 // bin of the nu = 1/2 column, one more partial sum per warp).
 // LZ: the adjoint of the Lanczos-shifted model (more tables, fewer resident
 // CTAs for the registers of the transposed convolution).
-template <int N, int CPG = 1, bool WN = false, bool LZ = false>
+template <int N, bool WN = false, bool LZ = false>
 struct BwdCfg {
   static constexpr int H = N / 2 + 1;
   static constexpr int TPF = N / 8;
   static constexpr int NFFT = N / 2;
-  static constexpr int GROUPS = NFFT / CPG;
-  static constexpr int THREADS = GROUPS * TPF;
-  static constexpr bool G_SMEM = CPG == 1;   // gradient patch staged in shared memory
+  static constexpr int THREADS = NFFT * TPF;
   static constexpr int WARPS = THREADS / 32;
   static constexpr int LS = psf_lstride(N);
   static constexpr int PSF_ELEMS = psf_spec_elems(N);
@@ -52,39 +45,38 @@ struct BwdCfg {
   // untangle as column k (lanes of a warp: 8 or more k, four groups' rows),
   // then transformed one per group.  Strides chosen against bank conflicts
   // of both patterns: N = 64 shifts rows 2-3 of every 4 by 4 float2 in an
-  // 88-float2 stride, N = 128 uses an odd stride.
+  // 88-float2 stride.
   static constexpr int WS = wstride<N>();
-  static constexpr int W_ELEMS = (CPG == 1 ? NFFT : GROUPS) * WS;
+  static constexpr int W_ELEMS = NFFT * WS;
   static constexpr int WSA = N == 64 ? 88 : N == 128 ? 129 : WS;
   static constexpr int SKEWA = N == 64 ? 4 : 0;
   static_assert(SKEWA <= WSA - WS, "shifted rows must not overlap");
   __host__ __device__ static constexpr int rowA(int r) { return r * WSA + SKEWA * ((r >> 1) & 1); }
   static constexpr int WA_ELEMS = NFFT * WSA;
-  // Gradient patch rows in shared memory (floats): N <= 64 pads them by 8 so
-  // that the row transforms' loads (rows p of four groups) hit distinct
-  // banks; N = 128 has no room and keeps them dense.
-  static constexpr int GS = N <= 64 ? N + 8 : N;
+  // Gradient patch rows in shared memory (floats), padded by 8 so that the row
+  // transforms' loads (rows p of four groups) hit distinct banks.
+  static constexpr int GS = N + 8;
   static constexpr int R1 = Radix<N>::r[1];
   static constexpr int R2 = Radix<N>::r[2];
   static constexpr int TW1 = twiddle_elems<N, R1>();
   static constexpr int TW2 = Radix<N>::P == 3 ? twiddle_elems<N, (R2 > 1 ? R2 : 2)>() : 0;
-  // Resident CTAs per SM: 10 (N = 32), 3 (N = 64), 1 (N = 128).  The PSF
+  // Resident CTAs per SM: 10 (N = 32), 4 (N = 64).  The PSF
   // spectrum is read from global memory (L2-resident) rather than staged in
   // shared memory, and the gradient patch is not prefetched a galaxy ahead:
   // both would take the shared memory that the extra resident CTAs need, and
   // more resident warps hide more latency (measured: 32 x 32 1.06 -> 1.02 ms,
   // 64 x 64 2.68 -> 2.11 ms per 100k).
-  static constexpr int MIN_BLOCKS = LZ ? (N == 32 ? 8 : N == 64 ? 3 : 1) : N == 32 ? 10 : N == 64 ? 4 : CPG;
+  static constexpr int MIN_BLOCKS = LZ ? (N == 32 ? 8 : 3) : N == 32 ? 10 : 4;
   // N = 64: the gradient patch and the row transforms' work rows share one
   // region (both 18 KB): the real-space pass and the row transforms' first
   // loads read the patch, then a CTA barrier, then the work rows are written
-  static constexpr bool ALIAS_G = N == 64 && CPG == 1;
+  static constexpr bool ALIAS_G = N == 64;
   static_assert(!ALIAS_G || sizeof(float) * N * GS <= sizeof(float2) * NFFT * WS, "patch must fit the work rows");
 
   static constexpr size_t off_wa = 0;
   static constexpr size_t off_wb = off_wa + sizeof(float2) * WA_ELEMS;
   static constexpr size_t off_g = ALIAS_G ? off_wb : (off_wb + sizeof(float2) * W_ELEMS + 15) & ~size_t(15);
-  static constexpr size_t off_tw = (ALIAS_G || !G_SMEM) ? off_wb + sizeof(float2) * W_ELEMS : off_g + sizeof(float) * N * GS;
+  static constexpr size_t off_tw = ALIAS_G ? off_wb + sizeof(float2) * W_ELEMS : off_g + sizeof(float) * N * GS;
   // (the shift phase along nu is computed where it is used, one value per
   // thread and column: no table)
   static constexpr int NYS = WN ? 4 : 3;   // nu = 1/2 column sums per bin: S, Sq, Sn (and Sd)
@@ -116,10 +108,10 @@ static_assert(4 * (BwdCfg<64>::SMEM + 512 + 1024) <= 196 * 1024, "64 x 64 adjoin
 // responses are folded into the phase tables, d/dx and d/dy are the values
 // through the slopes' responses, and the real-space terms (at the integer
 // offset) are contracted with the transposed convolution of the patch.
-template <int N, bool WN, bool EIG, bool LZ, int CPG = 1>
-__global__ void __launch_bounds__(BwdCfg<N, CPG, WN, LZ>::THREADS, BwdCfg<N, CPG, WN, LZ>::MIN_BLOCKS)
+template <int N, bool WN, bool EIG, bool LZ>
+__global__ void __launch_bounds__(BwdCfg<N, WN, LZ>::THREADS, BwdCfg<N, WN, LZ>::MIN_BLOCKS)
     render_bwd_kernel(RenderParams p, const float* __restrict__ grad_out, float* __restrict__ grad_params) {
-  using C = BwdCfg<N, CPG, WN, LZ>;
+  using C = BwdCfg<N, WN, LZ>;
   constexpr int TPF = C::TPF, WS = C::WS, LS = C::LS;
   constexpr int B = bucket_of(N);
   constexpr float INV_N = 1.0f / N;
@@ -188,9 +180,8 @@ __global__ void __launch_bounds__(BwdCfg<N, CPG, WN, LZ>::THREADS, BwdCfg<N, CPG
   // patch before this galaxy's writes, and only thread 0 (the final sums)
   // still reads anything of it, in program order before its own next writes.
   // For N = 32 one more after the record lands (the set-up tasks read the PSF
-  // mixture from shared memory); the larger sides read it from global memory
-  // (L2) instead (measured: 128 x 128 3.38 -> 3.17 ms, 64 x 64 2.10 -> 2.07
-  // ms with both barriers gone, 32 x 32 0.816 -> 0.835 without the second).
+  // mixture from shared memory); the other side reads it from global memory
+  // (L2) instead (measured: 64 x 64 2.10 -> 2.07 ms with both barriers gone, 32 x 32 0.816 -> 0.835 without the second).
   constexpr bool REC_SYNC = N == 32;
   __syncthreads();
   for (int buf = 0;; buf ^= 1) {
@@ -206,15 +197,11 @@ __global__ void __launch_bounds__(BwdCfg<N, CPG, WN, LZ>::THREADS, BwdCfg<N, CPG
     rec_parity ^= 1u << buf;
     const AdjRecord& r = rec[buf];
     const bool go = rec_landed && r.ok;
-    if (C::G_SMEM && go && warp == 0) {   // the gradient patch: one bulk copy per padded row, or one of the dense patch
-      if constexpr (C::GS == N) {
-        if (lane == 0) bulk_load(gbuf, grad_out + r.off, sizeof(float) * N * N, &bar[2]);
-      } else {
-        if (lane == 0) mbar_expect_tx(&bar[2], sizeof(float) * N * N);
-        __syncwarp();
-        for (int y = lane; y < N; y += 32)
-          bulk_copy(gbuf + y * C::GS, grad_out + r.off + (size_t)y * N, sizeof(float) * N, &bar[2]);
-      }
+    if (go && warp == 0) {   // the gradient patch: one bulk copy per padded row
+      if (lane == 0) mbar_expect_tx(&bar[2], sizeof(float) * N * N);
+      __syncwarp();
+      for (int y = lane; y < N; y += 32)
+        bulk_copy(gbuf + y * C::GS, grad_out + r.off + (size_t)y * N, sizeof(float) * N, &bar[2]);
     }
     if (go && r.psf != cur_psf) {
       const DevPsf& ps = p.psfs[r.psf];
@@ -320,11 +307,9 @@ __global__ void __launch_bounds__(BwdCfg<N, CPG, WN, LZ>::THREADS, BwdCfg<N, CPG
       }
     }
     bool g_landed = true;
-    if constexpr (C::G_SMEM) {
-      if (go) {
-        g_landed = mbar_wait(&bar[2], g_parity);
-        g_parity ^= 1u;
-      }
+    if (go) {
+      g_landed = mbar_wait(&bar[2], g_parity);
+      g_parity ^= 1u;
     }
     if (__syncthreads_or(!g_landed || !rec_landed)) {   // S2
       if (tid == 0) set_status(p.status, MOG_ERR_TIMEOUT);
@@ -333,22 +318,17 @@ __global__ void __launch_bounds__(BwdCfg<N, CPG, WN, LZ>::THREADS, BwdCfg<N, CPG
 
     float acc[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     float2 v[8];
-    // the gradient patch: staged in shared memory, or the caller's (L2)
-    const float* gsrc = C::G_SMEM ? gbuf : grad_out + r.off;
-    constexpr int GSTR = C::G_SMEM ? C::GS : N;
     if constexpr (C::ALIAS_G)   // the patch is read before the work rows overwrite it
-      adj_real_space<N, WN, LZ>(gsrc, GSTR, at, real_terms_padded(r.nrc * s_kpsf), tid, C::THREADS, acc, r.s11, r.s12,
+      adj_real_space<N, WN, LZ>(gbuf, C::GS, at, real_terms_padded(r.nrc * s_kpsf), tid, C::THREADS, acc, r.s11, r.s12,
                                 r.s22, s_lw);
     // ---- forward FFT of row pairs (prow, prow + N/2) packed as g[prow] + i g[prow + N/2] ----
-#pragma unroll 1
-    for (int rr = 0; rr < CPG; ++rr) {
-      const int prow = f + rr * C::GROUPS;
-      const float* ga = gsrc + prow * GSTR;
-      const float* gb = gsrc + (prow + N / 2) * GSTR;
+    {
+      const int prow = f;
+      const float* ga = gbuf + prow * C::GS;
+      const float* gb = gbuf + (prow + N / 2) * C::GS;
 #pragma unroll
       for (int m = 0; m < 8; ++m) v[m] = make_float2(ga[j + m * TPF], gb[j + m * TPF]);
       if constexpr (C::ALIAS_G) __syncthreads();   // every row of the patch is in registers
-      if (rr > 0) __syncwarp();   // the group's reads of its work row for the previous pair are done
       dft8<-1>(v);
 #pragma unroll
       for (int m = 0; m < 8; ++m) wb[swz<N>(8 * j + m)] = v[m];
@@ -378,13 +358,12 @@ __global__ void __launch_bounds__(BwdCfg<N, CPG, WN, LZ>::THREADS, BwdCfg<N, CPG
 
     // ---- real-space terms: analytic derivatives, pixel by pixel ----
     if constexpr (!C::ALIAS_G)
-      adj_real_space<N, WN, LZ>(gsrc, GSTR, at, real_terms_padded(r.nrc * s_kpsf), tid, C::THREADS, acc, r.s11, r.s12,
+      adj_real_space<N, WN, LZ>(gbuf, C::GS, at, real_terms_padded(r.nrc * s_kpsf), tid, C::THREADS, acc, r.s11, r.s12,
                                 r.s22, s_lw);
     __syncthreads();  // S3: every column input written
 
-#pragma unroll 1
-    for (int cc = 0; cc < CPG; ++cc) {
-      const int col = f + cc * C::GROUPS;   // column nu = col / N (column 0: nu = 0 and 1/2 packed)
+    {
+      const int col = f;   // column nu = col / N (column 0: nu = 0 and 1/2 packed)
       float2* wa = WA + C::rowA(col);
       // ---- forward FFT of every column along y ----
 #pragma unroll
@@ -424,12 +403,9 @@ __global__ void __launch_bounds__(BwdCfg<N, CPG, WN, LZ>::THREADS, BwdCfg<N, CPG
         // mixture sums at the thread's bins b = q R + m, components outer and
         // bins (2k, 2k+1) in packed f32x2, BH bins per sweep over the
         // components: N = 64 takes two sweeps of 4 (its register budget at
-        // four CTAs per SM), N = 128 four sweeps of 2 (64 registers for 1024
-        // threads: half the spills of two sweeps, 4.02 -> 3.95 ms for the
-        // 32.8k 128 x 128 galaxies of the mixed workload).  No warp-level skip
-        // of negligible components: the per-component vote cost more than the
-        // work it saved (measured).
-        constexpr int BH = N >= 128 ? 2 : N >= 64 ? 4 : 8;
+        // four CTAs per SM).  No warp-level skip of negligible components: the
+        // per-component vote cost more than the work it saved (measured).
+        constexpr int BH = N == 64 ? 4 : 8;
 #pragma unroll
         for (int b0 = 0; b0 < 8; b0 += BH) {
           float2 qp[BH / 2], S[BH / 2], SQ[BH / 2], SN[BH / 2], SD[BH / 2];
@@ -522,29 +498,20 @@ __global__ void __launch_bounds__(BwdCfg<N, CPG, WN, LZ>::THREADS, BwdCfg<N, CPG
   }
 }
 
-// Row pairs per group of the launched kernel: two at N = 128 (two 512-thread
-// CTAs per SM).
-template <int N>
-constexpr int bwd_cpg() { return N == 128 ? 2 : 1; }
-
-static_assert(2 * (BwdCfg<128, 2, true>::SMEM + 1024) <= 228 * 1024, "two 128 x 128 adjoint CTAs share an SM");
-
 template <int N, bool WN = false, bool EIG = false, bool LZ = false>
 static int bwd_occupancy() {
-  constexpr int CPG = bwd_cpg<N>();
-  using C = BwdCfg<N, CPG, WN, LZ>;
-  return kernel_occupancy(reinterpret_cast<const void*>(render_bwd_kernel<N, WN, EIG, LZ, CPG>), C::THREADS, C::SMEM);
+  using C = BwdCfg<N, WN, LZ>;
+  return kernel_occupancy(reinterpret_cast<const void*>(render_bwd_kernel<N, WN, EIG, LZ>), C::THREADS, C::SMEM);
 }
 
 template <int N, bool WN, bool EIG, bool LZ>
 static cudaError_t launch_bwd_mode(const RenderParams& p, const float* grad_out, float* grad_params, int num_sms,
                                    int ctas_per_sm, cudaStream_t s) {
-  constexpr int CPG = bwd_cpg<N>();
-  using C = BwdCfg<N, CPG, WN, LZ>;
+  using C = BwdCfg<N, WN, LZ>;
   const int occ = bwd_occupancy<N, WN, EIG, LZ>();
   if (occ < 0) return cudaErrorInvalidConfiguration;
   const int ctas = (ctas_per_sm > 0 && ctas_per_sm < occ) ? ctas_per_sm : occ;
-  render_bwd_kernel<N, WN, EIG, LZ, CPG><<<persistent_grid(p, ctas, num_sms), C::THREADS, C::SMEM, s>>>(p, grad_out, grad_params);
+  render_bwd_kernel<N, WN, EIG, LZ><<<persistent_grid(p, ctas, num_sms), C::THREADS, C::SMEM, s>>>(p, grad_out, grad_params);
   return cudaGetLastError();
 }
 
@@ -569,7 +536,7 @@ int render_bwd_max_ctas(int n) {
   switch (n) {
     case 32: return bwd_occupancy<32>();
     case 64: return bwd_occupancy<64>();
-    case 128: return bwd_occupancy<128>();
+    case 128: return render_bwd128_max_ctas();
     case 256: return 1;
     default: return 0;
   }
@@ -580,7 +547,7 @@ cudaError_t launch_render_bwd(int n, const RenderParams& p, const float* grad_ou
   switch (n) {
     case 32: return launch_bwd<32>(p, grad_out, grad_params, num_sms, ctas_per_sm, s);
     case 64: return launch_bwd<64>(p, grad_out, grad_params, num_sms, ctas_per_sm, s);
-    case 128: return launch_bwd<128>(p, grad_out, grad_params, num_sms, ctas_per_sm, s);
+    case 128: return launch_render_bwd128(p, grad_out, grad_params, num_sms, ctas_per_sm, s);
     default: return cudaErrorInvalidValue;
   }
 }

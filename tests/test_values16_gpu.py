@@ -77,13 +77,14 @@ def test_parity_with_skipped_galaxies(gpu_renderer, tables, mode, size, count, b
 
 
 @pytest.mark.parametrize("sersic", [False, True])
-@pytest.mark.parametrize("count,bad", [(1, None), (3, 1), (41, 38), (300, 297)])
-def test_adjoint_parity_with_skipped_galaxies(gpu_renderer, tables, sersic, count, bad):
+@pytest.mark.parametrize("size,count,bad", [(256, 1, None), (256, 3, 1), (256, 41, 38), (256, 300, 297),
+                                            (128, 1, None), (128, 3, 1), (128, 400, 397)])
+def test_adjoint_parity_with_skipped_galaxies(gpu_renderer, tables, sersic, size, count, bad):
     import torch
     from paper_2012_15797_gb300 import capi
     from paper_2012_15797_gb300.renderer import to_device
     from oracle import adjoint as A
-    gals = _batch(count, bad)
+    gals = _batch(count, bad, size)
     b = to_device(gals)
     go = torch.randn(b.total, generator=torch.Generator(device="cuda").manual_seed(count), device="cuda")
     gp = torch.full((count, 7 if sersic else 6), 7.0, device="cuda")
@@ -100,8 +101,8 @@ def test_adjoint_parity_with_skipped_galaxies(gpu_renderer, tables, sersic, coun
             continue
         g = gals.row(i)
         psf = gpu_renderer.psfs[g["psf"]]
-        pix = go[int(b.offsets[i]):int(b.offsets[i]) + 256 * 256].double().cpu().numpy().reshape(256, 256)
-        hat = R.psf_spectrum(psf.image, 256)
+        pix = go[int(b.offsets[i]):int(b.offsets[i]) + size * size].double().cpu().numpy().reshape(size, size)
+        hat = R.psf_spectrum(psf.image, size)
         want = A.vjp(g, hat, psf.mog, tables, pix)
         norm = np.abs(pix).sum()
         scale = np.array([1.0] + [abs(g["flux"])] * 5)
@@ -111,16 +112,16 @@ def test_adjoint_parity_with_skipped_galaxies(gpu_renderer, tables, sersic, coun
             assert abs(got[i, 6] - dn) <= 1e-4 * abs(dn) + 1e-5 * norm * abs(g["flux"]), i
 
 
-@pytest.mark.parametrize("count", [1, 41, 300])
-def test_lanczos_adjoint_small_and_large_batches(gpu_renderer, tables, count):
+@pytest.mark.parametrize("size,count", [(256, 1), (256, 41), (256, 300), (128, 1), (128, 400)])
+def test_lanczos_adjoint_small_and_large_batches(gpu_renderer, tables, size, count):
     import torch
     from paper_2012_15797_gb300.renderer import to_device
     from test_lanczos_adjoint_gpu import check, oracle_grads_lanczos
-    gals = _batch(count, None)
+    gals = _batch(count, None, size)
     b = to_device(gals)
     go = torch.randn(b.total, generator=torch.Generator(device="cuda").manual_seed(count), device="cuda")
     got = gpu_renderer.render_backward(b, go, shift="lanczos")
-    last = [go[int(b.offsets[-1]):].double().cpu().numpy().reshape(256, 256)]
+    last = [go[int(b.offsets[-1]):].double().cpu().numpy().reshape(size, size)]
     one = gals.subset(np.array([count - 1]))
     check(got[-1:].double().cpu().numpy(), oracle_grads_lanczos(one, gpu_renderer.psfs, tables, last), one, last)
     gals.x[:] = np.round(gals.x * 4)
