@@ -39,7 +39,8 @@ UNIT = "patches/s"
 PARAM_BYTES = 7 * 4 + 3 * 4 + 8      # float params, int ids, int64 offset
 SFU_PER_CLK_SM = 32                  # MUFU ex2 per SM per clock (measured live: "pipe_rates" in the line)
 FP32_FLOP_PER_CLK_SM = 256           # 128 FMA lanes x 2 (measured live: "pipe_rates")
-KERNEL_SOURCES = ("paper_2012_15797_gb300/csrc/render_fwd.cu", "paper_2012_15797_gb300/csrc/common.cuh")
+KERNEL_SOURCES = tuple("paper_2012_15797_gb300/csrc/" + f
+                       for f in ("render_fwd64.cu", "fwd16.cuh", "fft16.cuh", "common.cuh"))
 PROFILE_SUMMARY = os.path.join(ROOT, "profiles", "render_fwd_64_100k.md")
 KERNELS_PER_RENDER = 5   # the planner's three kernels, the record prologue, the size kernel
 
@@ -489,7 +490,7 @@ def extra_mixed(tables, device, steps, pk, cpu_seconds=0.0):
     # kernel against its own galaxies' work over its event time
     kpsf = psfs[0].mog.shape[0]
     res["roofline"] = roofline(algorithmic_work(gals, tables, kpsf), graph_ms, pk,
-                               "graph: render_fwd_kernel<32|64|128> + render_fwd256_kernel")
+                               "graph: render_fwd_kernel<32> + render_fwd64|128|256_kernel")
     # each size's kernel alone (batch size mask = that side), CUDA events
     # around its launches: its own time and roofline
     per = {}
@@ -594,7 +595,7 @@ def extra_render_grad(tables, psf, device, steps, pk, cpu_seconds=0.0):
            "kernel_ms_forward": fwd_ms, "kernel_ms_adjoint": bwd_ms,
            "roofline": roofline(wb, bwd_ms, pk, "render_bwd_kernel<64>"),
            "roofline_forward_plus_adjoint_kernels": roofline(add_work(wf, wb), fwd_ms + bwd_ms, pk,
-                                                             "render_fwd_kernel<64> + render_bwd_kernel<64>")}
+                                                             "render_fwd64_kernel + render_bwd_kernel<64>")}
     # the plain form: one render-with-loss and one adjoint call per galaxy, on 2000 of them
     singles = [to_device(model.subset([i]), device=dev) for i in range(2000)]
     g1 = torch.empty(64 * 64, device=dev)
@@ -1194,7 +1195,7 @@ def run_ours(args):
     pk = peaks(props.multi_processor_count)
     work = algorithmic_work(gals, tables, psf.mog.shape[0])
     k_ms = kms[1] / max(kn[1], 1)
-    roof = roofline(work, k_ms, pk, "render_fwd_kernel<64>", traffic=recorded_traffic(args.galaxies))
+    roof = roofline(work, k_ms, pk, "render_fwd64_kernel", traffic=recorded_traffic(args.galaxies))
 
     cpu = None
     if world == 1 and not args.no_cpu:
@@ -1223,7 +1224,7 @@ def run_ours(args):
         "real_space_component_fraction": work["real_fraction"],
         "roofline": roof, "cpu_baseline": cpu, "e2e": e2e,
         # per step: plan_histogram, plan_scan, plan_scatter, galaxy_prep and
-        # render_fwd_kernel<64> (the launch list in profiles/render_fwd_64_100k.md)
+        # render_fwd64_kernel (the launch list in profiles/render_fwd_64_100k.md)
         "gpu_launches": args.steps * KERNELS_PER_RENDER, "clocks": clocks, "pipe_rates": pipes,
         "extra": extra,
     }

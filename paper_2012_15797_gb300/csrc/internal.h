@@ -124,6 +124,8 @@ int kernel_occupancy(const void* fn, int threads, size_t smem);
 // schedule (composites when p.records2 is set).
 cudaError_t launch_render_fwd128(const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s);
 int render_fwd128_max_ctas();
+cudaError_t launch_render_fwd64(const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s);
+int render_fwd64_max_ctas();
 cudaError_t launch_render_fwd(int n, const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s);
 // Composites (mog_render_composite): one transform per galaxy for the two
 // profiles of p.records and p.records2 (N = 32, 64, 128; and 256).

@@ -686,9 +686,15 @@ static cudaError_t launch_fwd(const RenderParams& p, int num_sms, int ctas_per_s
     return p.lanczos ? launch_fwd_mode<N, true, true, 0>(p, num_sms, ctas_per_sm, s)
                      : launch_fwd_mode<N, false, true, 0>(p, num_sms, ctas_per_sm, s);
   if (p.lanczos) return launch_fwd_mode<N, true, false, 0>(p, num_sms, ctas_per_sm, s);
-  if (N == 64 && p.sched == 2) return launch_render_fwd64w(p, num_sms, ctas_per_sm, s);
   return p.sched == 1 ? launch_fwd_mode<N, false, false, 1>(p, num_sms, ctas_per_sm, s)
                       : launch_fwd_mode<N, false, false, 0>(p, num_sms, ctas_per_sm, s);
+}
+
+// 64 x 64: the first schedule is render_fwd64.cu's, the third render_fwd64w.cu's.
+static cudaError_t launch_fwd_64(const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s) {
+  if (p.sched == 0 || p.loss || p.eigen || p.lanczos) return launch_render_fwd64(p, num_sms, ctas_per_sm, s);
+  return p.sched == 2 ? launch_render_fwd64w(p, num_sms, ctas_per_sm, s)
+                      : launch_fwd_mode<64, false, false, 1>(p, num_sms, ctas_per_sm, s);
 }
 
 // 128 x 128: the first schedule is render_fwd128.cu's.
@@ -716,7 +722,7 @@ cudaError_t launch_render_fwd_composite(int n, const RenderParams& p, int num_sm
 cudaError_t launch_render_fwd(int n, const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s) {
   switch (n) {
     case 32: return launch_fwd<32>(p, num_sms, ctas_per_sm, s);
-    case 64: return launch_fwd<64>(p, num_sms, ctas_per_sm, s);
+    case 64: return launch_fwd_64(p, num_sms, ctas_per_sm, s);
     case 128: return launch_fwd_128(p, num_sms, ctas_per_sm, s);
     case 256: return launch_render_fwd256(p, num_sms, ctas_per_sm, s);
     default: return cudaErrorInvalidValue;
@@ -727,7 +733,7 @@ int render_fwd_max_ctas(int n, int sched) {
   switch (n) {
     case 32: return sched == 1 ? fwd_occupancy<32, false, false, 1>() : fwd_occupancy<32>();
     case 64: return sched == 2 ? render_fwd64w_max_ctas()
-                  : sched == 1 ? fwd_occupancy<64, false, false, 1>() : fwd_occupancy<64>();
+                  : sched == 1 ? fwd_occupancy<64, false, false, 1>() : render_fwd64_max_ctas();
     case 128: return sched == 2   ? fwd_occupancy<128, false, false, 2>()
                      : sched == 1 ? fwd_occupancy<128, false, false, 1>() : render_fwd128_max_ctas();
     case 256: return render_fwd256_max_ctas(sched);

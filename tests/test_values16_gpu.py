@@ -1,4 +1,4 @@
-"""The kernels with 16 values per thread (256 x 256, 128 x 128) against the FP64
+"""The kernels with 16 values per thread (256 x 256, 128 x 128, 64 x 64) against the FP64
 oracle, with a galaxy that is skipped in the middle.  Forward, every mode: batch
 sizes around the pipeline depth (tables one galaxy ahead, records three ahead),
 for 256 x 256 below and above the line from which a CTA and no longer a cluster
@@ -31,7 +31,8 @@ def _batch(count, bad, size=256):
 
 @pytest.mark.parametrize("mode", ["phase", "lanczos", "loss", "composite"])
 @pytest.mark.parametrize("size,count,bad", [(256, 1, None), (256, 2, 0), (256, 3, 1), (256, 7, 3), (256, 640, 637),
-                                            (128, 1, None), (128, 2, 0), (128, 3, 1), (128, 640, 637)])
+                                            (128, 1, None), (128, 2, 0), (128, 3, 1), (128, 640, 637),
+                                            (64, 1, None), (64, 2, 0), (64, 3, 1), (64, 640, 637)])
 def test_parity_with_skipped_galaxies(gpu_renderer, tables, mode, size, count, bad):
     import torch
     from paper_2012_15797_gb300 import capi
@@ -135,7 +136,7 @@ def test_lanczos_adjoint_small_and_large_batches(gpu_renderer, tables, size, cou
 
 
 @pytest.mark.parametrize("mode", ["phase", "lanczos"])
-@pytest.mark.parametrize("size", [128, 256])
+@pytest.mark.parametrize("size", [64, 128, 256])
 def test_adding_to_an_image_is_the_image_plus_the_model(gpu_renderer, mode, size):
     import torch
     from paper_2012_15797_gb300.renderer import to_device
@@ -144,4 +145,34 @@ def test_adding_to_an_image_is_the_image_plus_the_model(gpu_renderer, mode, size
     out = base.clone()
     gpu_renderer.render(b, out, shift=mode, add=True)
     assert torch.equal(out, base + gpu_renderer.render(b, shift=mode))
+    gpu_renderer.sync_status()
+
+
+@pytest.mark.parametrize("chunk", [1, 3])
+@pytest.mark.parametrize("mode", ["phase", "lanczos"])
+def test_psfs_that_change_from_galaxy_to_galaxy(gpu_renderer, mode, chunk):
+    """64 x 64, few galaxies of each of five PSFs per CTA (one CTA per SM), the
+    first of a PSF skipped now and then: the bits of every galaxy by itself."""
+    import torch
+    from paper_2012_15797_gb300 import capi
+    from paper_2012_15797_gb300.renderer import patches, to_device
+    count = 1500
+    gals = _batch(count, None, 64)
+    gals.psf[:] = np.arange(count) % 5
+    gals.flux[::211] = np.nan
+    capi.mog_set_launch_shape(gpu_renderer.ctx, 0, 64, 1, chunk, 0)
+    try:
+        b = to_device(gals)
+        out = gpu_renderer.render(b, torch.zeros(b.total, device="cuda"), shift=mode)
+        with pytest.raises(capi.MogError):
+            gpu_renderer.sync_status()
+    finally:
+        capi.mog_set_launch_shape(gpu_renderer.ctx, 0, 64, 0, 1, 0)
+    got = patches(out, b)
+    for i in range(1, count, 37):
+        if np.isnan(gals.flux[i]):
+            continue
+        one = to_device(gals.subset(np.array([i])))
+        alone = patches(gpu_renderer.render(one, shift=mode), one)[0]
+        assert torch.equal(got[i], alone), i
     gpu_renderer.sync_status()
