@@ -124,6 +124,7 @@ int kernel_occupancy(const void* fn, int threads, size_t smem);
 // schedule (composites when p.records2 is set).
 cudaError_t launch_render_fwd128(const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s);
 int render_fwd128_max_ctas();
+// 64 x 64 likewise (render_fwd64.cu; no composites).
 cudaError_t launch_render_fwd64(const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s);
 int render_fwd64_max_ctas();
 cudaError_t launch_render_fwd(int n, const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s);
