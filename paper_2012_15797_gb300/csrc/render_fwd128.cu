@@ -21,8 +21,8 @@
 // memory 53%, FMA pipe 48%).  Against 8 values per thread (two exchanges per
 // transform, two 512-thread CTAs at 64 registers, tables made between barriers):
 // the 32.8k 128 x 128 galaxies of the 200k mixed workload 1.72 -> 1.50 ms (with
-// the loss 2.00 -> 1.84, Lanczos 2.97 -> 2.67, composites 2.22 -> 2.16, eigen-PSFs
-// 2.76 -> 1.99).
+// the loss 2.00 -> 1.84, composites 2.22 -> 2.16, eigen-PSFs 2.76 -> 1.99; a call
+// with the Lanczos shift on 32.8k galaxies of one profile 2.30 -> 1.75).
 #include "fwd16.cuh"
 
 namespace mog {

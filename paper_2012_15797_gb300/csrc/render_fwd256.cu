@@ -26,7 +26,8 @@
 // barriers per round, 512 threads at 64 registers): 129k warp instructions and
 // 18k shared-memory wavefronts per galaxy instead of 199k and 43k; the 10.6k
 // 256 x 256 galaxies of the 200k mixed workload 2.47 -> 2.00 ms (with the loss
-// 2.83 -> 2.68, Lanczos 4.09 -> 3.52, composites 2.94 -> 2.65 ms).
+// 2.83 -> 2.68, composites 2.94 -> 2.65 ms; a call with the Lanczos shift on 10.6k
+// galaxies of one profile 2.97 -> 2.31).
 //
 // Lanczos variant (LZ): the Fourier part is shifted through the phase tables
 // (the Lanczos transfer function H(nu) H(omega)); a galaxy with real-space
