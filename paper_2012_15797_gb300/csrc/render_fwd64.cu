@@ -19,7 +19,8 @@
 // 2.2k shared-memory wavefronts per galaxy; 100k galaxies 0.976 -> 0.935 ms, the
 // call 1.039 -> 0.998 (1.068 with the PSF spectrum read through L1, 1.018 with it in shared
 // memory at four CTAs, 1.065 at five with the twiddles in registers, spilled),
-// the fit step of 50k 1.671 -> 1.641, 40k of an eigen-PSF 0.695 -> 0.662.
+// the fit step of 50k 1.671 -> 1.641, 40k of an eigen-PSF 0.695 -> 0.662; with the
+// Lanczos shift (four CTAs) 30k 0.419 -> 0.421, 300 galaxies 36 -> 29 us.
 #include "fwd16.cuh"
 
 namespace mog {
