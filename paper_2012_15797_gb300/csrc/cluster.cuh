@@ -11,9 +11,10 @@ __device__ __forceinline__ uint32_t cluster_rank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
+// Every arrival releases: a thread's reads of another CTA's shared memory, too,
+// are ordered before that CTA's next writes only by release and acquire (a
+// relaxed arrival orders nothing, also after the loads' values have been used).
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
-// Arrival that orders no memory: for readers whose loads have returned.
-__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 
 // Address in the shared memory of CTA `rank` of the cluster of the location

@@ -404,9 +404,9 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) render_fwd256c_kernel(Re
         __syncwarp();   // the group's previous reads of its work row are done
         fft16<N, +1>(
             tw, v, [&](int k1) { return w + k1 * EX + j; }, [&](int q, int i) { return w + j * EX + i; }, [&] {
-          // C2: the thread's last gathers have returned (the exchange's
-          // writes, issued before, depend on all of them)
-          if (rr == ROUNDS - 1) cluster_arrive_relaxed();
+          // C2: the thread's last gathers have been issued before (the
+          // exchange's writes depend on all of them)
+          if (rr == ROUNDS - 1) cluster_arrive();
         });
         __syncwarp();
         float* const orow = reinterpret_cast<float*>(w);
