@@ -718,6 +718,23 @@ __device__ __forceinline__ float2 lanczos_response(const float (&w)[7], float f)
   return make_float2(re, im);
 }
 
+// The same of the weights' slopes w'_a, whose sum is zero (the weights' is one):
+// H'(f) = sum_a w'_a (z^a - 1), with cos(a theta) - 1 = -2 sin^2(a theta / 2).
+// The sum of w'_a z^a cancels from terms of order one to one of order f, and
+// what FP32 leaves of the slopes' sum goes, times the galaxy's whole value, into
+// its gradient: here the response is exact to rounding down to f = 0.  (w[3] is
+// not used.)
+__device__ __forceinline__ float2 lanczos_slope_response(const float (&w)[7], float f) {
+  float s, c;
+  sincospif(f, &s, &c);                      // half the angle
+  const float h2 = 2.0f * s * c, h3 = s * fmaf(-4.0f * s, s, 3.0f);   // sin 2, 3 times it
+  const float c1 = fmaf(-2.0f * s, s, 1.0f);
+  const float s2 = 2.0f * h2 * c1, s3 = h2 * fmaf(-4.0f * h2, h2, 3.0f);   // sin of the angle: h2, of 2, 3 times it
+  const float re = -2.0f * fmaf(w[6] + w[0], h3 * h3, fmaf(w[5] + w[1], h2 * h2, (w[4] + w[2]) * s * s));
+  const float im = -fmaf(w[6] - w[0], s3, fmaf(w[5] - w[1], s2, (w[4] - w[2]) * h2));
+  return make_float2(re, im);
+}
+
 // Record of the adjoint (Section 2 Steps 3-4 plus the derivatives the
 // gradient needs).  With e_i = 2^(fcoef_i q):
 //   S  = sum famp_i e_i                  (spectrum value, as in the forward)
@@ -1111,7 +1128,8 @@ __device__ __forceinline__ void contract_bin(float2 z, float nu, float om, float
 }
 
 // Lanczos weights of the adjoint, per galaxy: w along x at [0, 7), their slopes
-// dw/dd at [8, 15), the same along y at [16, 23) and [24, 31).
+// dw/dd at [8, 15), the same along y at [16, 23) and [24, 31).  The slopes add
+// up to zero exactly (lanczos_adj.cuh).
 constexpr int ADJ_LW = 32;
 
 // The transposed periodic Lanczos convolutions of the upstream gradient g at 8

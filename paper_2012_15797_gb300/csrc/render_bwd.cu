@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(BwdCfg<N, WN, LZ>::THREADS, BwdCfg<N, WN, LZ>:
             if (l < ADJ_LW) s_lw[l] = lwg[l];
             float w[7];
             load_weights(lwg, 24, w);
-            pyd[l] = cmul(py[l], lanczos_response(w, om));
+            pyd[l] = cmul(py[l], lanczos_slope_response(w, om));
             load_weights(lwg, 16, w);
             py[l] = cmul(py[l], lanczos_response(w, om));
           }
@@ -279,11 +279,11 @@ __global__ void __launch_bounds__(BwdCfg<N, WN, LZ>::THREADS, BwdCfg<N, WN, LZ>:
             load_weights(lwg, 0, w);
             const float2 hx = cmul(bx, lanczos_response(w, 0.5f));
             load_weights(lwg, 8, w);
-            const float2 hxd = cmul(bx, lanczos_response(w, 0.5f));
+            const float2 hxd = cmul(bx, lanczos_slope_response(w, 0.5f));
             load_weights(lwg, 16, w);
             const float2 hy = cmul(by, lanczos_response(w, om));
             load_weights(lwg, 24, w);
-            const float2 hyd = cmul(by, lanczos_response(w, om));
+            const float2 hyd = cmul(by, lanczos_slope_response(w, om));
             nyb[l] = cmul(pn, cmul(hx, hy));
             nybx[l] = cmul(pn, cmul(hxd, hy));
             nyby[l] = cmul(pn, cmul(hx, hyd));
@@ -395,7 +395,7 @@ __global__ void __launch_bounds__(BwdCfg<N, WN, LZ>::THREADS, BwdCfg<N, WN, LZ>:
           float w[7];
 #pragma unroll
           for (int a = 0; a < 7; ++a) w[a] = s_lw[8 + a];
-          pxd = cmul(pxf, lanczos_response(w, (float)col * INV_N));
+          pxd = cmul(pxf, lanczos_slope_response(w, (float)col * INV_N));
 #pragma unroll
           for (int a = 0; a < 7; ++a) w[a] = s_lw[a];
           pxf = cmul(pxf, lanczos_response(w, (float)col * INV_N));

@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
           if constexpr (LZ) {
             float w[7];
             load_weights(lwg, 24, w);
-            phyd = cmul(phy, lanczos_response(w, om));
+            phyd = cmul(phy, lanczos_slope_response(w, om));
             load_weights(lwg, 16, w);
             phy = cmul(phy, lanczos_response(w, om));
           }
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
             if constexpr (LZ) {
               float w[7];
               load_weights(lwg, 8, w);
-              phxd = cmul(phx, lanczos_response(w, 0.5f));
+              phxd = cmul(phx, lanczos_slope_response(w, 0.5f));
               load_weights(lwg, 0, w);
               phx = cmul(phx, lanczos_response(w, 0.5f));
             }
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
           if constexpr (LZ) {
             float w[7];
             load_weights(lwg, 8, w);
-            pxd[k] = cmul(ph, lanczos_response(w, (float)k * INV_N));
+            pxd[k] = cmul(ph, lanczos_slope_response(w, (float)k * INV_N));
             load_weights(lwg, 0, w);
             ph = cmul(ph, lanczos_response(w, (float)k * INV_N));
           }

@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(THREADS, LZ ? 1 : CTAS_PER_SM)
             if (i < ADJ_LW) s_lw[i] = lwg[i];
             float wv[7];
             load_weights(lwg, 8, wv);
-            pxd[i] = cmul(px[i], lanczos_response(wv, (float)i * INV_N));
+            pxd[i] = cmul(px[i], lanczos_slope_response(wv, (float)i * INV_N));
             load_weights(lwg, 0, wv);
             px[i] = cmul(px[i], lanczos_response(wv, (float)i * INV_N));
           }
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(THREADS, LZ ? 1 : CTAS_PER_SM)
           if constexpr (LZ) {
             float wv[7];
             load_weights(lwg, 24, wv);
-            pyd[l] = cmul(py[l], lanczos_response(wv, om));
+            pyd[l] = cmul(py[l], lanczos_slope_response(wv, om));
             load_weights(lwg, 16, wv);
             py[l] = cmul(py[l], lanczos_response(wv, om));
           }
@@ -210,11 +210,11 @@ __global__ void __launch_bounds__(THREADS, LZ ? 1 : CTAS_PER_SM)
             load_weights(lwg, 0, wv);
             const float2 hx = cmul(bx, lanczos_response(wv, 0.5f));
             load_weights(lwg, 8, wv);
-            const float2 hxd = cmul(bx, lanczos_response(wv, 0.5f));
+            const float2 hxd = cmul(bx, lanczos_slope_response(wv, 0.5f));
             load_weights(lwg, 16, wv);
             const float2 hy = cmul(by, lanczos_response(wv, om));
             load_weights(lwg, 24, wv);
-            const float2 hyd = cmul(by, lanczos_response(wv, om));
+            const float2 hyd = cmul(by, lanczos_slope_response(wv, om));
             nyb[l] = cmul(pn, cmul(hx, hy));
             nybx[l] = cmul(pn, cmul(hxd, hy));
             nyby[l] = cmul(pn, cmul(hx, hyd));

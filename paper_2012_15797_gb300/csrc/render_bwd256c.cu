@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     auto shift = [&](float2 ph, int at, float fr, float2& slope) {
       float wv[7];
       load_weights(lwg, at + 8, wv);
-      slope = cmul(ph, lanczos_response(wv, fr));
+      slope = cmul(ph, lanczos_slope_response(wv, fr));
       load_weights(lwg, at, wv);
       return cmul(ph, lanczos_response(wv, fr));
     };
