@@ -9,6 +9,7 @@
 #include <utility>
 #include <vector>
 
+#include "branches.h"
 #include "ctx.h"
 
 using namespace mog;
@@ -425,18 +426,21 @@ template <class Launch>
 mog_status launch_buckets(mog_ctx* ctx, Workspace* ws, const mog_batch* batch, uint32_t supported, cudaStream_t s,
                           bool largest_first, Launch&& launch) {
   const uint32_t want = batch->size_mask ? (batch->size_mask & supported) : supported;
-  const bool fork = __builtin_popcount(want) > 1 && !ctx->serial_buckets;
-  if (fork) MOG_CUDA(ctx, cudaEventRecord(ws->fork_ev, s));
-  const int last = !want ? 0 : largest_first ? __builtin_ctz(want) : 31 - __builtin_clz(want);
+  const bool parallel = __builtin_popcount(want) > 1 && !ctx->serial_buckets;
+  int order[NBUCKET], n = 0;
   for (int i = 0; i < NBUCKET; ++i) {
     const int b = largest_first ? NBUCKET - 1 - i : i;
-    if (!((want >> b) & 1)) continue;
-    const bool side = fork && b != last;
-    cudaStream_t bs = s;
-    if (side) {
-      bs = ws->side[b];
-      MOG_CUDA(ctx, cudaStreamWaitEvent(bs, ws->fork_ev, 0));
-    }
+    if ((want >> b) & 1) order[n++] = b;
+  }
+  if (parallel) MOG_CUDA(ctx, cudaEventRecord(ws->fork_ev, s));
+  auto side = [&](int i) { return parallel && i < n - 1; };
+  auto fork = [&](int i) -> mog_status {
+    if (side(i)) MOG_CUDA(ctx, cudaStreamWaitEvent(ws->side[order[i]], ws->fork_ev, 0));
+    return MOG_OK;
+  };
+  auto run = [&](int i) -> mog_status {
+    const int b = order[i];
+    const cudaStream_t bs = side(i) ? ws->side[b] : s;
     mog_ctx::Timed t{b, nullptr, nullptr};
     if (ctx->timing) {
       MOG_CUDA(ctx, take_event(ctx, &t.a));
@@ -448,12 +452,16 @@ mog_status launch_buckets(mog_ctx* ctx, Workspace* ws, const mog_batch* batch, u
       MOG_CUDA(ctx, cudaEventRecord(t.b, bs));
       ctx->pending.push_back(t);
     }
-    if (side) MOG_CUDA(ctx, cudaEventRecord(ws->join_ev[b], bs));
-  }
-  if (fork)
-    for (int b = 0; b < NBUCKET; ++b)
-      if (((want >> b) & 1) && b != last) MOG_CUDA(ctx, cudaStreamWaitEvent(s, ws->join_ev[b], 0));
-  return MOG_OK;
+    return MOG_OK;
+  };
+  auto join = [&](int i) -> mog_status {
+    if (side(i)) {
+      MOG_CUDA(ctx, cudaEventRecord(ws->join_ev[order[i]], ws->side[order[i]]));
+      MOG_CUDA(ctx, cudaStreamWaitEvent(s, ws->join_ev[order[i]], 0));
+    }
+    return MOG_OK;
+  };
+  return run_branches<mog_status>(n, MOG_OK, fork, run, join);
 }
 
 }  // namespace
