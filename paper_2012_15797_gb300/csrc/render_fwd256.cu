@@ -262,6 +262,10 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) render_fwd256_kernel(Ren
     // patch holds, this CTA's slice of the workspace scratch
     float2* const zbuf = p.accumulate ? p.scratch256 + (size_t)blockIdx.x * (N / 2) * N
                                       : reinterpret_cast<float2*>(p.out + off);
+    // Lanczos and adding to the patch: the Fourier part of a galaxy with
+    // real-space terms stays there until they are convolved (the model is added
+    // to the patch as a whole)
+    const bool park = LZ && p.accumulate != 0 && nrt > 0;
 
     // ---- Steps 5-6 on the bins l = j + m T of each of the group's columns, Step 7a ----
     float2 v[16];
@@ -381,7 +385,7 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) render_fwd256_kernel(Ren
           d[N] = z.y;
         }
         __syncwarp();   // the group's two rows are complete
-        float* const dst = p.out + off + (size_t)pr * N;
+        float* const dst = (park ? reinterpret_cast<float*>(zbuf) : p.out + off) + (size_t)pr * N;
 #pragma unroll 1
         for (int i = 0; i < 2; ++i) {
           const int x0 = 8 * (j + T * i), p0 = x0 ^ cx ^ (((x0 >> 5) & 1) << 2);
@@ -402,7 +406,7 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) render_fwd256_kernel(Ren
             for (int u = 0; u < 8; ++u) ov[u] = h ? o[u].y : o[u].x;
             if constexpr (LOSS)
               chi += loss_store8(dat, p.out + off, mdl, (int64_t)(pr + h * (N / 2)) * N + x0, ov, 2.0f * iv);
-            else store8(dst + h * (N / 2) * N + x0, ov, p.accumulate != 0);
+            else store8(dst + h * (N / 2) * N + x0, ov, p.accumulate != 0 && !park);
           }
         }
       }
@@ -418,14 +422,16 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) render_fwd256_kernel(Ren
     }
     if constexpr (LZ) {
       if (nrt > 0) {   // uniform
-        __syncthreads();   // the whole Fourier part is in the patch; W is free
+        __syncthreads();   // the whole Fourier part is in the patch (or parked); W is free
         float* const dst = p.out + off;
+        const float* const src = park ? reinterpret_cast<const float*>(zbuf) : dst;
         lanczos_real_strips<N, STRIP, THREADS>(
             rt, nrt, s_lzw[LZ ? buf : 0], reinterpret_cast<float*>(smem), [&](int y, int x0, const float(&acc)[8]) {
-              float4* const d = reinterpret_cast<float4*>(dst + y * N + x0);
+              const float4* const d = reinterpret_cast<const float4*>(src + y * N + x0);
               const float4 f0 = d[0], f1 = d[1];   // the Fourier part, written by this CTA
-              d[0] = make_float4(f0.x + acc[0], f0.y + acc[1], f0.z + acc[2], f0.w + acc[3]);
-              d[1] = make_float4(f1.x + acc[4], f1.y + acc[5], f1.z + acc[6], f1.w + acc[7]);
+              const float ov[8] = {f0.x + acc[0], f0.y + acc[1], f0.z + acc[2], f0.w + acc[3],
+                                   f1.x + acc[4], f1.y + acc[5], f1.z + acc[6], f1.w + acc[7]};
+              store8(dst + y * N + x0, ov, park);
             });
       }
     }

@@ -249,11 +249,9 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) render_fwd256c_kernel(Re
   // Before C1(i): the columns of i (reading its Fourier tables and record),
   // the Fourier tables of i + 1 (buffer (i + 1) & 1, last read before
   // C1(i - 1); from the record of i + 1, loaded before C1(i - 1)), the
-  // real-space terms of i (buffer i & 1, last read by the rows of i - 2; with
-  // one CTA per galaxy one buffer, written after C2(i - 1)) and
+  // real-space terms of i (buffer i & 1, last read by the rows of i - 2) and
   // the record of i + 2 (the buffer of i - 1, last read before C1(i - 1)).
-  // The rows use no record: what they need of it is in registers.  With one
-  // CTA per galaxy a CTA barrier at the wait's place stands for C2.
+  // The rows use no record: what they need of it is in registers.
   bool pending = false;   // an arrival at C2 whose wait is still to come
   int b3 = 0;
   for (int buf = 0; pos >= 0; buf ^= 1) {
@@ -535,12 +533,9 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) render_fwd256c_kernel(Re
           const float* const src = park ? parked + (size_t)(pl + (rr & 1) * KL) * N : dst;
           float F[2][8];
 #pragma unroll
-          for (int i = 0; i < 2; ++i) {
-            const float4* d = reinterpret_cast<const float4*>(src + 8 * (j + T * i));
-            const float4 a = d[0], b = d[1];   // written by this thread
-            F[i][0] = a.x; F[i][1] = a.y; F[i][2] = a.z; F[i][3] = a.w;
-            F[i][4] = b.x; F[i][5] = b.y; F[i][6] = b.z; F[i][7] = b.w;
-          }
+          for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int u = 0; u < 8; ++u) F[i][u] = 0.0f;
 #pragma unroll 1
           for (int b = -3; b <= 3; ++b) {
             const int row = (y - b) & (N - 1), rp = row & (N / 2 - 1);
@@ -554,8 +549,16 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) render_fwd256c_kernel(Re
               for (int u = 0; u < 8; ++u) F[i][u] = fmaf(wb, t[u], F[i][u]);
             }
           }
+          // added to the Fourier part at the end, as in lanczos_real_strips: the
+          // two kernels of this side round alike
 #pragma unroll
-          for (int i = 0; i < 2; ++i) store8(dst + 8 * (j + T * i), F[i], park);
+          for (int i = 0; i < 2; ++i) {
+            const float4* d = reinterpret_cast<const float4*>(src + 8 * (j + T * i));
+            const float4 a = d[0], b = d[1];   // written by this thread
+            const float o[8] = {a.x + F[i][0], a.y + F[i][1], a.z + F[i][2], a.w + F[i][3],
+                                b.x + F[i][4], b.y + F[i][5], b.z + F[i][6], b.w + F[i][7]};
+            store8(dst + 8 * (j + T * i), o, park);
+          }
         }
         cluster_arrive();   // C2 again: the gathers of these rows are done
       }

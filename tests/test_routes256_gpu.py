@@ -1,0 +1,119 @@
+"""256 x 256 galaxies: the kernel of a few (a cluster of CTAs per galaxy) and the
+one of many (a CTA per galaxy) are chosen by how many there are, so a galaxy has
+to have the same bits from both, in every mode.  Batches above the lines between
+them (8 galaxies per SM; 0.75 for the adjoint, 1.5 with the Lanczos shift), with
+galaxies that are skipped, against the batch of their first galaxies, and against
+the FP64 oracle with the tolerances of the parity tests (render: max |d pixel| <=
+2e-6 flux; gradients: 1e-4 |g| + 1e-5 ||dL/dpix||_1 s)."""
+
+import numpy as np
+import pytest
+
+from oracle import eigenpsf as E
+from oracle import lanczos as L
+from oracle import render as R
+from workloads import eigen_positions
+from test_eigenpsf_gpu import eig, eig_renderer   # noqa: F401  (fixtures)
+from test_values16_gpu import _batch
+
+pytestmark = pytest.mark.gpu
+
+FEW = 24          # galaxies of the small batch
+SKIPPED = (3, 20)  # galaxies with a parameter that is not finite
+MANY = 3200
+N = 256
+
+
+@pytest.fixture
+def renderer(request, gpu_renderer, eig_renderer):   # noqa: F811
+    return {"constant": gpu_renderer, "eigen": eig_renderer}[request.param]
+
+
+def _galaxies(count, eigen):
+    gals = _batch(count, None, N)
+    gals.log_re[::3] = np.log(40.0)   # some with real-space terms
+    gals.profile[::6] = 1
+    gals.sersic_n[::6] = 4.0
+    gals.flux[list(SKIPPED)] = np.nan
+    gals.flux[count - 2] = np.nan
+    if eigen:
+        gals.psf[:] = 1
+    return gals, (eigen_positions(count, seed=91) if eigen else None)
+
+
+def _reference(gals, pos, i, shift, renderer, eig, tables):   # noqa: F811
+    g = gals.row(i)
+    if pos is not None:
+        img, mog = E.psf_at(eig, float(pos[0][i]), float(pos[1][i]))
+    else:
+        img, mog = renderer.psfs[g["psf"]].image, renderer.psfs[g["psf"]].mog
+    return (L.render_lanczos if shift == "lanczos" else R.render)(g, img, mog, tables)
+
+
+def _sub(gals, pos):
+    few = np.arange(FEW)
+    return gals.subset(few), (None if pos is None else (pos[0][:FEW], pos[1][:FEW]))
+
+
+def _status(r):
+    from paper_2012_15797_gb300 import capi
+    with pytest.raises(capi.MogError):
+        r.sync_status()
+
+
+@pytest.mark.parametrize("shift", ["phase", "lanczos"])
+@pytest.mark.parametrize("renderer,eigen,mode", [   # (composites take constant PSFs)
+    ("constant", False, "render"), ("constant", False, "add"), ("constant", False, "composite"),
+    ("eigen", True, "render"), ("eigen", True, "add")], indirect=["renderer"])
+def test_renders(renderer, eig, tables, eigen, mode, shift):   # noqa: F811
+    import torch
+    from paper_2012_15797_gb300.renderer import patches, to_device
+    count = MANY
+    gals, pos = _galaxies(count, eigen)
+    base = torch.randn(count * N * N, generator=torch.Generator(device="cuda").manual_seed(7), device="cuda")
+
+    def run(g, q):
+        b = to_device(g, positions=q)
+        out = base[:b.total].clone()
+        if mode == "composite":
+            renderer.render_composite(b, b, out, shift=shift)
+        else:
+            renderer.render(b, out, shift=shift, add=mode == "add")
+        _status(renderer)
+        return out, b
+
+    many, b = run(gals, pos)
+    few, bf = run(*_sub(gals, pos))
+    assert torch.equal(many[:few.numel()], few)
+    skipped = [*SKIPPED, count - 2]
+    got, before = patches(many, b), patches(base, b)
+    if mode == "add":
+        plain = torch.zeros_like(base)
+        renderer.render(b, plain, shift=shift)
+        _status(renderer)
+        assert torch.equal(many, base + plain)
+    for i in skipped:
+        assert torch.equal(got[i], before[i])
+    for i in [*range(7), *range(count - 4, count)]:
+        if i in skipped:
+            continue
+        flux = float(gals.flux[i]) * (2.0 if mode == "composite" else 1.0)
+        ref = _reference(gals, pos, i, shift, renderer, eig, tables) * (2.0 if mode == "composite" else 1.0)
+        img = got[i].double().cpu().numpy()
+        if mode == "add":   # (the sum is rounded to the pixel that was there)
+            img, tol = img - before[i].double().cpu().numpy(), 2e-6 * flux + 3e-7 * float(before[i].abs().max())
+        else:
+            tol = 2e-6 * flux
+        assert np.max(np.abs(img - ref)) <= tol, i
+
+
+def test_lanczos_batches_in_host_memory(gpu_renderer):
+    """Chunks below the line between the kernels, the same bits as one call above it."""
+    import torch
+    from paper_2012_15797_gb300.renderer import host_batch, to_device
+    gals = _batch(MANY, None, N)
+    gals.log_re[::3] = np.log(40.0)
+    want = gpu_renderer.render(to_device(gals), shift="lanczos")
+    got = gpu_renderer.render_host(host_batch(gals), torch.empty(want.numel()), shift="lanczos")
+    gpu_renderer.sync_status()
+    assert torch.equal(want.cpu(), got)
