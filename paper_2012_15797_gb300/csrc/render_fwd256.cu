@@ -53,6 +53,7 @@ constexpr int PSF_ELEMS = psf_spec_elems(N);
 constexpr int B = bucket_of(N);
 constexpr int HALF = N / 2 + 2;            // omega = 0 .. 1/2 (padded)
 constexpr int STRIP = 64;                  // Lanczos: output rows per strip
+constexpr int CHI_SUMS = ROUNDS / 2 * WARPS;
 
 // float2 offset of element c of row pair p's transform input in the patch
 __device__ __forceinline__ int zpos(int p, int c) { return (c < N / 2 ? p : p + N / 2) * (N / 2) + (c & (N / 2 - 1)); }
@@ -107,7 +108,7 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) render_fwd256_kernel(Ren
   RT& rt = *reinterpret_cast<RT*>(smem + C::off_rt);
   __shared__ int s_first[3], s_pos[2];
   __shared__ float s_lzw[LZ ? 2 : 1][16];   // per buffer: Lanczos weights along x [0, 7) and y [8, 15)
-  __shared__ float s_chi[LOSS ? 2 : 1][WARPS];   // each warp's sum of squared residuals
+  __shared__ float s_chi[LOSS ? 2 : 1][LOSS ? CHI_SUMS : 1];   // sums of squared residuals: [rounds 2 i, 2 i + 1][warp]
 
   const int tid = threadIdx.x;
   const int f = tid / T, j = tid % T;
@@ -149,7 +150,7 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) render_fwd256_kernel(Ren
   auto write_chi2 = [&]() {
     if (chi_gal >= 0) {
       float t = 0.0f;
-      for (int i = 0; i < WARPS; ++i) t += s_chi[chi_buf][i];
+      for (int i = 0; i < CHI_SUMS; ++i) t += s_chi[chi_buf][i];
       p.chi2[chi_gal] = chi_iv * t;
       chi_gal = -1;
     }
@@ -409,10 +410,17 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) render_fwd256_kernel(Ren
             else store8(dst + h * (N / 2) * N + x0, ov, p.accumulate != 0 && !park);
           }
         }
+        if constexpr (LOSS) {
+          // every two rounds (32 row pairs) have a sum per warp: the order in
+          // which the cluster kernel, a CTA for each 32, adds them
+          if (rr & 1) {
+            for (int o2 = 16; o2 > 0; o2 >>= 1) chi += __shfl_xor_sync(0xffffffffu, chi, o2);
+            if ((tid & 31) == 0) s_chi[LOSS ? buf : 0][(rr >> 1) * WARPS + (tid >> 5)] = chi;
+            chi = 0.0f;
+          }
+        }
       }
       if constexpr (LOSS) {
-        for (int o2 = 16; o2 > 0; o2 >>= 1) chi += __shfl_xor_sync(0xffffffffu, chi, o2);
-        if ((tid & 31) == 0) s_chi[LOSS ? buf : 0][tid >> 5] = chi;
         if (tid == 0) {
           chi_gal = gal;
           chi_iv = iv;

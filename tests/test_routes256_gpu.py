@@ -117,3 +117,39 @@ def test_lanczos_batches_in_host_memory(gpu_renderer):
     got = gpu_renderer.render_host(host_batch(gals), torch.empty(want.numel()), shift="lanczos")
     gpu_renderer.sync_status()
     assert torch.equal(want.cpu(), got)
+
+
+@pytest.mark.parametrize("renderer,eigen", [("constant", False), ("eigen", True)], indirect=["renderer"])
+def test_loss(renderer, eig, tables, eigen):   # noqa: F811
+    """Pixels, gradient patches and chi^2, whose sum has one order in both kernels."""
+    import torch
+    from paper_2012_15797_gb300.renderer import patches, to_device
+    count = MANY
+    gals, pos = _galaxies(count, eigen)
+    data = torch.randn(count * N * N, generator=torch.Generator(device="cuda").manual_seed(8), device="cuda")
+    ivar = torch.rand(count, generator=torch.Generator(device="cuda").manual_seed(9), device="cuda") + 0.5
+
+    def run(g, q):
+        b = to_device(g, positions=q)
+        grad = torch.full((b.total,), 7.0, device="cuda")
+        model = torch.full((b.total,), 7.0, device="cuda")
+        _, chi2 = renderer.render_chi2(b, data[:b.total], ivar[:b.count], grad, model=model)
+        _status(renderer)
+        return b, grad, model, chi2
+
+    b, grad, model, chi2 = run(gals, pos)
+    _, fgrad, fmodel, fchi2 = run(*_sub(gals, pos))
+    assert torch.equal(grad[:fgrad.numel()], fgrad) and torch.equal(model[:fmodel.numel()], fmodel)
+    assert torch.equal(chi2[:FEW].nan_to_num(-1.0), fchi2.nan_to_num(-1.0))
+    skipped = [*SKIPPED, count - 2]
+    assert sorted(torch.nonzero(torch.isnan(chi2))[:, 0].tolist()) == skipped
+    pg, pm, pd = patches(grad, b), patches(model, b), patches(data, b)
+    for i in [*range(7), *range(count - 4, count)]:
+        if i in skipped:
+            assert bool((pg[i] == 7.0).all()) and bool((pm[i] == 7.0).all())
+            continue
+        ref = _reference(gals, pos, i, "phase", renderer, eig, tables)
+        assert np.max(np.abs(pm[i].double().cpu().numpy() - ref)) <= 2e-6 * float(gals.flux[i]), i
+        assert torch.equal(pg[i], 2.0 * ivar[i] * (pm[i] - pd[i]))
+        want = float(ivar[i]) * np.sum((ref - pd[i].double().cpu().numpy()) ** 2)
+        assert abs(float(chi2[i]) - want) <= 1e-5 * want, i
