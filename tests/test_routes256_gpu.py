@@ -153,3 +153,79 @@ def test_loss(renderer, eig, tables, eigen):   # noqa: F811
         assert torch.equal(pg[i], 2.0 * ivar[i] * (pm[i] - pd[i]))
         want = float(ivar[i]) * np.sum((ref - pd[i].double().cpu().numpy()) ** 2)
         assert abs(float(chi2[i]) - want) <= 1e-5 * want, i
+
+
+@pytest.mark.parametrize("shift", ["phase", "lanczos"])
+@pytest.mark.parametrize("sersic", [False, True])
+@pytest.mark.parametrize("renderer,eigen", [("constant", False), ("eigen", True)], indirect=["renderer"])
+def test_adjoint(renderer, eig, tables, eigen, sersic, shift):   # noqa: F811
+    import torch
+    from oracle import adjoint as A
+    from paper_2012_15797_gb300.renderer import to_device
+    count = 400   # more than there are CTAs, so that some take two galaxies
+    gals, pos = _galaxies(count, eigen)
+    go = torch.randn(count * N * N, generator=torch.Generator(device="cuda").manual_seed(10), device="cuda") + 0.25
+
+    def run(g, q):
+        b = to_device(g, positions=q)
+        gp = torch.full((b.count, 7 if sersic else 6), 7.0, device="cuda")
+        renderer.render_backward(b, go[:b.total].contiguous(), gp, sersic=sersic, shift=shift)
+        _status(renderer)
+        return gp
+
+    many, few = run(gals, pos), run(*_sub(gals, pos))
+    assert torch.equal(many[:FEW], few)
+    skipped = [*SKIPPED, count - 2]
+    for i in [*range(7), *range(count - 4, count)]:
+        if i in skipped:
+            assert bool((many[i] == 7.0).all())
+            continue
+        g = gals.row(i)
+        if g["e1"] == 0.0 and g["e2"] == 0.0:   # not differentiable by e1, e2
+            continue
+        if eigen:
+            img, mog = E.psf_at(eig, float(pos[0][i]), float(pos[1][i]))
+        else:
+            img, mog = renderer.psfs[g["psf"]].image, renderer.psfs[g["psf"]].mog
+        pix = go[i * N * N:(i + 1) * N * N].double().cpu().numpy().reshape(N, N)
+        hat = R.psf_spectrum(img, N)
+        want = (L.vjp_lanczos if shift == "lanczos" else A.vjp)(g, hat, mog, tables, pix)
+        if sersic:
+            dn = (L.sersic_derivative_lanczos if shift == "lanczos" else A.sersic_derivative)(g, hat, mog, tables)
+            want = np.append(want, np.sum(dn * pix))
+        scale = np.array([1.0] + [abs(g["flux"])] * (len(want) - 1)) * np.abs(pix).sum()
+        got = many[i].double().cpu().numpy()
+        assert np.all(np.abs(got - want) <= 1e-4 * np.abs(want) + 1e-5 * scale), (i, got, want)
+
+
+def test_served_alone_and_in_a_micro_batch(gpu_renderer):
+    """Requests of a few 256 x 256 galaxies among others, one micro-batch each
+    and in micro-batches of hundreds: the same gradients and chi^2."""
+    from paper_2012_15797_gb300.serving import Server, make_fits
+    from workloads import mixed_galaxies
+    gals = _batch(400, None, N)
+    gals.size[::5] = mixed_galaxies(80, seed=92, n_psf=1).size
+    gals.log_re[:] = np.minimum(gals.log_re, np.log(gals.size / 8.0)).astype(np.float32)
+    state = make_fits(gpu_renderer, [gals])
+    rng = np.random.default_rng(93)
+    reqs = []
+    for _ in range(12):
+        c = int(rng.integers(1, 60))
+        first = int(rng.integers(0, len(gals) - c + 1))
+        p = gals.params6()[first:first + c].copy()
+        p[:, 0] *= 1.0 + 0.05 * rng.standard_normal(c)
+        reqs.append((0, first, p.astype(np.float32)))
+    got = []
+    for most in (0, 4096):
+        srv = Server(gpu_renderer, budget_bytes=1 << 30, lanes=1, max_batch_galaxies=most)
+        srv.add_fit(**state[0])
+        tickets, keeps = srv.replay(reqs, np.zeros(len(reqs)))
+        srv.wait_replayed(tickets, keeps)
+        stats = srv.stats()
+        assert (stats["batches"] == len(reqs)) == (most == 0)
+        srv.close()
+        got.append([(k[1].copy(), k[2].copy()) for k in keeps])
+    for (g0, c0), (g1, c1) in zip(*got):
+        assert np.all(np.isfinite(g0)) and np.all(np.isfinite(c0))
+        np.testing.assert_array_equal(g0, g1)
+        np.testing.assert_array_equal(c0, c1)
