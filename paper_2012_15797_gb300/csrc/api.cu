@@ -68,6 +68,9 @@ cudaError_t workspace_init(Workspace* ws) {
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ws->join_ev[b], cudaEventDisableTiming);
   }
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ws->fork_ev, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&ws->side256.s, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ws->side256.fork, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ws->side256.join, cudaEventDisableTiming);
   return e;
 }
 
@@ -87,6 +90,9 @@ void workspace_free(Workspace* ws) {
     if (ws->join_ev[b]) cudaEventDestroy(ws->join_ev[b]);
   }
   if (ws->fork_ev) cudaEventDestroy(ws->fork_ev);
+  if (ws->side256.s) cudaStreamDestroy(ws->side256.s);
+  if (ws->side256.fork) cudaEventDestroy(ws->side256.fork);
+  if (ws->side256.join) cudaEventDestroy(ws->side256.join);
   *ws = Workspace{};
 }
 
@@ -400,7 +406,6 @@ mog_status batch_params(mog_ctx* ctx, Workspace* ws, const mog_batch* batch, flo
   *p = RenderParams{};
   p->b = view_of(batch);
   p->max_galaxies = batch->count;
-  p->only_side = batch->size_mask && !(batch->size_mask & (batch->size_mask - 1)) ? 1 : 0;
   p->out = out;
   p->profiles = ctx->d_profiles;
   p->psfs = ctx->d_psfs;
@@ -501,7 +506,7 @@ mog_status render_with(mog_ctx* ctx, Workspace* ws, const mog_batch* batch, floa
     RenderParams q = p;
     q.chunk = ctx->tune_fwd[bucket_of(n)].chunk;
     q.sched = ctx->tune_fwd[bucket_of(n)].sched;
-    return launch_render_fwd(n, q, ctx->num_sms, ctx->tune_fwd[bucket_of(n)].ctas_per_sm, bs);
+    return launch_render_fwd(n, q, ctx->num_sms, ctx->tune_fwd[bucket_of(n)].ctas_per_sm, bs, &ws->side256);
   });
 }
 
@@ -533,7 +538,7 @@ mog_status backward_with(mog_ctx* ctx, Workspace* ws, const mog_batch* batch, co
   return launch_buckets(ctx, ws, batch, BWD_BUCKETS, s, false, [&](int n, cudaStream_t bs) {
     RenderParams q = p;
     q.chunk = ctx->tune_bwd[bucket_of(n)].chunk;
-    if (n == 256) return launch_render_bwd256(q, grad_out, grad_params, ws->bwd256, ctx->num_sms, bs);
+    if (n == 256) return launch_render_bwd256(q, grad_out, grad_params, ws->bwd256, ctx->num_sms, bs, &ws->side256);
     return launch_render_bwd(n, q, grad_out, grad_params, ctx->num_sms, ctx->tune_bwd[bucket_of(n)].ctas_per_sm, bs);
   });
 }
@@ -614,7 +619,7 @@ mog_status mog_render_composite(mog_ctx* ctx, const mog_batch* first, const mog_
     const LaunchShape& ls = ctx->tune_fwd[bucket_of(n)];
     q.chunk = ls.chunk;
     q.sched = 0;
-    if (n == 256) return launch_render_fwd256_composite(q, ctx->num_sms, ls.ctas_per_sm, bs);
+    if (n == 256) return launch_render_fwd256_composite(q, ctx->num_sms, ls.ctas_per_sm, bs, &ws->side256);
     return launch_render_fwd_composite(n, q, ctx->num_sms, ls.ctas_per_sm, bs);
   });
 }
@@ -715,10 +720,30 @@ mog_status mog_autotune(mog_ctx* ctx, const mog_batch* batch, float* out, const 
       const int n_side = bucket_side(b);
       LaunchShape best = tune[b];
       double best_ms = 1e300;
-      for (int sched = 0; sched < (dir == 0 ? schedules_of(n_side) : 1); ++sched) {
+      // 256 x 256: one schedule, and where the kernel of few galaxies is the one
+      // that runs, the CTAs per SM (and, in the adjoint, the chunk) change
+      // nothing: they stay at what the kernel of many takes by itself
+      bool few = false;
+      if (n_side == 256) {
+        ctx->timing = false;
+        st = dir == 0 ? mog_render_batch(ctx, &one, out, stream)
+                      : mog_render_backward(ctx, &one, grad_out, grad_params, stream);
+        ctx->timing = timing_was;
+        if (st != MOG_OK) return st;
+        int32_t here = 0;
+        const cudaStream_t s = static_cast<cudaStream_t>(stream);
+        MOG_CUDA(ctx, cudaMemcpyAsync(&here, ctx->ws.plan.small + NBUCKET + b, sizeof(here), cudaMemcpyDeviceToHost, s));
+        MOG_CUDA(ctx, cudaStreamSynchronize(s));
+        const int line = dir == 0 ? few256_render(ctx->num_sms) : few256_adjoint(false, ctx->num_sms);
+        const int far = dir == 0 ? far256_render(ctx->num_sms) : far256_adjoint(ctx->num_sms);
+        few = here <= line && batch->count <= far;
+      }
+      const int scheds = dir == 0 && n_side != 256 ? schedules_of(n_side) : 1;
+      for (int sched = 0; sched < scheds; ++sched) {
         const int max_ctas = dir == 0 ? render_fwd_max_ctas(n_side, sched) : render_bwd_max_ctas(n_side);
-        for (int c = 1; c <= max_ctas; ++c)
+        for (int c = few ? max_ctas : 1; c <= max_ctas; ++c)
           for (int ch : chunks) {
+            if (few && dir == 1 && ch != chunks[0]) continue;
             tune[b].ctas_per_sm = c;
             tune[b].chunk = ch;
             tune[b].sched = sched;

@@ -26,6 +26,7 @@ struct Workspace {
   cudaStream_t side[NBUCKET] = {};
   cudaEvent_t fork_ev = nullptr;
   cudaEvent_t join_ev[NBUCKET] = {};
+  SideStream side256;                    // the 256 x 256 kernel of few galaxies beside that of many
 };
 
 cudaError_t workspace_init(Workspace* ws);

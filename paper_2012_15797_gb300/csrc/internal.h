@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "common.cuh"
+#include "routes.h"
 
 namespace mog {
 
@@ -23,7 +24,9 @@ struct RenderParams {
   int* status;
   int chunk;                    // queue positions taken per request
   int64_t max_galaxies = INT64_MAX;   // upper bound of the bucket's galaxies (the batch's count): no more CTAs
-  int only_side = 0;            // 1: the batch names a single patch side (all its galaxies are in this bucket)
+  // 256 x 256: the kernel returns at once unless the bucket's count, which the
+  // plan leaves on the device, is in this range (launch_by_count)
+  int bucket_min = 0, bucket_max = INT32_MAX;
   int lanczos = 0;              // 1: sub-pixel shift by Lanczos convolution
   float* lzw = nullptr;         // lanczos: 16 floats per planned position, weights along x [0, 7), y [8, 15);
                                 // adjoint: ADJ_LW floats, weights and slopes
@@ -61,6 +64,42 @@ struct PlanScratch {
   int32_t* order;    // [capacity]
 };
 
+// The most galaxies of the 256 x 256 kernels of few (routes.h; reasons and
+// figures at the kernels of many).
+inline int few256_render(int num_sms) { return 8 * num_sms; }
+inline int few256_adjoint(bool lanczos, int num_sms) { return (lanczos ? 6 : 3) * num_sms / 4; }
+// The most galaxies in a batch for which both are launched.  (Of the population
+// that a survey has, about one in twenty is 256 x 256: there these are at or
+// above the line.)
+inline int far256_render(int num_sms) { return 128 * num_sms; }
+inline int far256_adjoint(int num_sms) { return 16 * num_sms; }
+
+// A stream beside the caller's and the events that fork it from there and join
+// it back: where the two 256 x 256 kernels are launched side by side.  Without
+// one they follow one another.
+struct SideStream {
+  cudaStream_t s = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
+};
+template <class Few, class Many>
+cudaError_t launch_by_count(const RenderParams& p, int line, int far, cudaStream_t s, const SideStream* side, Few&& few,
+                            Many&& many) {
+  return launch_by_count(
+      p, line, far, cudaSuccess,
+      [&]() -> cudaError_t {
+        if (!side) return cudaSuccess;
+        const cudaError_t e = cudaEventRecord(side->fork, s);
+        return e == cudaSuccess ? cudaStreamWaitEvent(side->s, side->fork, 0) : e;
+      },
+      [&](const RenderParams& q, bool beside) { return few(q, beside && side ? side->s : s); },
+      [&](const RenderParams& q) { return many(q, s); },
+      [&]() -> cudaError_t {
+        if (!side) return cudaSuccess;
+        const cudaError_t e = cudaEventRecord(side->join, side->s);
+        return e == cudaSuccess ? cudaStreamWaitEvent(s, side->join, 0) : e;
+      });
+}
+
 // Up to this many galaxies the plan and the records are one launch that counts
 // each galaxy's position over the batch (plan_and_records): quadratic, 2.6 us of
 // warp instructions at 2048, against three more launches of the counting sort
@@ -92,7 +131,7 @@ int render_bwd128_max_ctas();
 // render_bwd256_scratch_bytes(num_sms) of global scratch, one slice per CTA.
 size_t render_bwd256_scratch_bytes(int num_sms);
 cudaError_t launch_render_bwd256(const RenderParams& p, const float* grad_out, float* grad_params, float2* scratch,
-                                 int num_sms, cudaStream_t s);
+                                 int num_sms, cudaStream_t s, const SideStream* side);
 
 // The same adjoint (phase shift) with a cluster of CTAs per galaxy, for few
 // galaxies; needs no scratch.
@@ -127,12 +166,15 @@ int render_fwd128_max_ctas();
 // 64 x 64 likewise (render_fwd64.cu; no composites).
 cudaError_t launch_render_fwd64(const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s);
 int render_fwd64_max_ctas();
-cudaError_t launch_render_fwd(int n, const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s);
+cudaError_t launch_render_fwd(int n, const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s,
+                              const SideStream* side = nullptr);
 // Composites (mog_render_composite): one transform per galaxy for the two
 // profiles of p.records and p.records2 (N = 32, 64, 128; and 256).
 cudaError_t launch_render_fwd_composite(int n, const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s);
-cudaError_t launch_render_fwd256_composite(const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s);
-cudaError_t launch_render_fwd256(const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s);
+cudaError_t launch_render_fwd256_composite(const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s,
+                                           const SideStream* side);
+cudaError_t launch_render_fwd256(const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s,
+                                 const SideStream* side);
 // Resident CTAs per SM of the plain forward kernel for side n and radix
 // schedule `sched` (what the autotuner searches up to).
 int render_fwd_max_ctas(int n, int sched);

@@ -101,6 +101,7 @@ __global__ void __launch_bounds__(CTA_THREADS, 1)
   float2 tw[15];
   fft16_twiddles<N>(j, tw);
   const int count = p.bucket_count[B], first = p.bucket_start[B];
+  if (count < p.bucket_min || count > p.bucket_max) return;   // the other kernel's (launch_by_count)
   const unsigned char* records = p.records + (size_t)first * sizeof(AdjRecord);
   int q_next = 0, q_end = 0, q_ahead = 0;
   auto next_position = [&]() -> int {
@@ -218,17 +219,8 @@ size_t render_bwd256_scratch_bytes(int num_sms) {
   return sizeof(float2) * (size_t)2 * num_sms * (N / 2) * N;
 }
 
-cudaError_t launch_render_bwd256(const RenderParams& p, const float* grad_out, float* grad_params, float2* scratch,
-                                 int num_sms, cudaStream_t s) {
-  // Few galaxies: a cluster per galaxy (render_bwd256c.cu): 10 galaxies 92 -> 29
-  // us (Lanczos 106 -> 42), 100 143 -> 81 (118 -> 124), about equal at 160 (205
-  // -> 241): a CTA of this kernel takes 90 to 140 us for one, and a cluster has
-  // an SM per CTA.  The line is the batch's count; in a batch of several sides
-  // about one in twenty is 256 x 256 (1000 galaxies: Lanczos 177 -> 154 us, 4000:
-  // 413 -> 465).  One line for both shifts: at integer offsets they give the
-  // same gradients.
-  if (p.max_galaxies <= (p.only_side ? 128 : 2560))
-    return launch_render_bwd256_small(p, grad_out, grad_params, num_sms, s);
+static cudaError_t launch_many(const RenderParams& p, const float* grad_out, float* grad_params, float2* scratch,
+                               int num_sms, cudaStream_t s) {
   auto fn = p.lanczos ? (p.eigen ? (p.grad_n ? render_bwd256_kernel<true, true, true> : render_bwd256_kernel<false, true, true>)
                                  : (p.grad_n ? render_bwd256_kernel<true, false, true> : render_bwd256_kernel<false, false, true>))
                       : (p.eigen ? (p.grad_n ? render_bwd256_kernel<true, true, false> : render_bwd256_kernel<false, true, false>)
@@ -237,6 +229,23 @@ cudaError_t launch_render_bwd256(const RenderParams& p, const float* grad_out, f
   if (kernel_occupancy(reinterpret_cast<const void*>(fn), CTA_THREADS, smem) < 0) return cudaErrorInvalidConfiguration;
   fn<<<persistent_grid(p, 1, num_sms), CTA_THREADS, smem, s>>>(p, grad_out, grad_params, scratch);
   return cudaGetLastError();
+}
+
+// Few galaxies: a cluster per galaxy (render_bwd256c.cu).  Up to one galaxy per SM
+// the call takes as long as one CTA for one, 85 to 100 us (Lanczos 120 to 150); the
+// clusters, 38 at a time, take 23 us (31) for each 38.  Calls on clusters and on
+// this kernel, 114 galaxies: 93 and 101 us (with the Sersic index 105 and 111), 152:
+// 115 and 87; Lanczos, 228: 206 and 211, 266: 233 and 226.
+cudaError_t launch_render_bwd256(const RenderParams& p, const float* grad_out, float* grad_params, float2* scratch,
+                                 int num_sms, cudaStream_t s, const SideStream* side) {
+  return launch_by_count(
+      p, few256_adjoint(p.lanczos != 0, num_sms), far256_adjoint(num_sms), s, side,
+      [&](const RenderParams& q, cudaStream_t qs) {
+        return launch_render_bwd256_small(q, grad_out, grad_params, num_sms, qs);
+      },
+      [&](const RenderParams& q, cudaStream_t qs) {
+        return launch_many(q, grad_out, grad_params, scratch, num_sms, qs);
+      });
 }
 
 }  // namespace mog

@@ -86,6 +86,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   auto at_k1 = [&](int k1) { return w + k1 * EX + j; };
   auto at_i = [&](int, int i) { return w + j * EX + i; };
   const int count = p.bucket_count[B], first = p.bucket_start[B];
+  if (count < p.bucket_min || count > p.bucket_max) return;   // the other kernel's (launch_by_count), for the whole cluster
   auto sync_all = [&]() {
     cluster_arrive();
     cluster_wait();

@@ -719,12 +719,13 @@ cudaError_t launch_render_fwd_composite(int n, const RenderParams& p, int num_sm
   }
 }
 
-cudaError_t launch_render_fwd(int n, const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s) {
+cudaError_t launch_render_fwd(int n, const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s,
+                              const SideStream* side) {
   switch (n) {
     case 32: return launch_fwd<32>(p, num_sms, ctas_per_sm, s);
     case 64: return launch_fwd_64(p, num_sms, ctas_per_sm, s);
     case 128: return launch_fwd_128(p, num_sms, ctas_per_sm, s);
-    case 256: return launch_render_fwd256(p, num_sms, ctas_per_sm, s);
+    case 256: return launch_render_fwd256(p, num_sms, ctas_per_sm, s, side);
     default: return cudaErrorInvalidValue;
   }
 }

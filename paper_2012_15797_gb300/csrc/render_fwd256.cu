@@ -116,6 +116,7 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) render_fwd256_kernel(Ren
   fft16_twiddles<N>(j, tw);
   const int cx = (f & 1) * T;   // staged output rows, see below
   const int count = p.bucket_count[B];
+  if (count < p.bucket_min || count > p.bucket_max) return;   // the other kernel's (launch_by_count)
   const int first = p.bucket_start[B];          // planned position of this bucket's first galaxy
   const unsigned char* records = p.records + (size_t)first * RECORD_BYTES;
   [[maybe_unused]] const unsigned char* records2 = COMP ? p.records2 + (size_t)first * RECORD_BYTES : nullptr;
@@ -476,34 +477,39 @@ static cudaError_t launch_fwd256(const RenderParams& p, int num_sms, int ctas_pe
 // Few galaxies: a cluster per galaxy (render_fwd256c.cu).  A CTA of this kernel
 // takes about 80 us for a galaxy, so below a few hundred galaxies the call takes
 // that long however few they are (10: 64 us on the earlier 512-thread CTAs, 30
-// on clusters; 400: 175 and 110), and up to a few thousand the last, partly
-// filled wave still weighs more than the clusters' lower rate (plain 0.206 us a
-// galaxy against 0.188, Lanczos 0.39 against 0.33).  The line is the batch's
-// count, the bucket's being known on the device only: with one side named it is
-// the bucket's, otherwise about one galaxy in twenty is 256 x 256.
-static bool few_galaxies(const RenderParams& p) {
-  const int64_t line = (p.lanczos || p.records2) ? 1500 : 3000;
-  return p.max_galaxies <= (p.only_side ? line : 16 * line);
-}
-
-cudaError_t launch_render_fwd256_composite(const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s) {
-  if (few_galaxies(p)) return launch_render_fwd256_small(p, num_sms, s);
-  return p.lanczos ? launch_fwd256<true, false, false, true>(p, num_sms, ctas_per_sm, s)
-                   : launch_fwd256<false, false, false, true>(p, num_sms, ctas_per_sm, s);
+// on clusters), and up to four rounds of its 304 CTAs the last, partly filled one
+// weighs more than the clusters' lower rate: calls of 1000 galaxies on clusters
+// 239 us against 269 (Lanczos 325 against 361, composites 304 against 327), of
+// 1500 339 against 331 (463 against 452, 436 against 402), of 3000 630 against
+// 587 (845 against 764, 817 against 729).
+cudaError_t launch_render_fwd256_composite(const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s,
+                                           const SideStream* side) {
+  return launch_by_count(
+      p, few256_render(num_sms), far256_render(num_sms), s, side,
+      [&](const RenderParams& q, cudaStream_t qs) { return launch_render_fwd256_small(q, num_sms, qs); },
+      [&](const RenderParams& q, cudaStream_t qs) {
+        return q.lanczos ? launch_fwd256<true, false, false, true>(q, num_sms, ctas_per_sm, qs)
+                         : launch_fwd256<false, false, false, true>(q, num_sms, ctas_per_sm, qs);
+      });
 }
 
 int render_fwd256_max_ctas(int) { return fwd256_occupancy<false, false, false, false>(); }
 
-cudaError_t launch_render_fwd256(const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s) {
-  if (few_galaxies(p)) return launch_render_fwd256_small(p, num_sms, s);
-  if (p.loss)
-    return p.eigen ? launch_fwd256<false, true, true>(p, num_sms, ctas_per_sm, s)
-                   : launch_fwd256<false, false, true>(p, num_sms, ctas_per_sm, s);
-  if (p.eigen)
-    return p.lanczos ? launch_fwd256<true, true>(p, num_sms, ctas_per_sm, s)
-                     : launch_fwd256<false, true>(p, num_sms, ctas_per_sm, s);
-  return p.lanczos ? launch_fwd256<true, false>(p, num_sms, ctas_per_sm, s)
-                   : launch_fwd256<false, false>(p, num_sms, ctas_per_sm, s);
+cudaError_t launch_render_fwd256(const RenderParams& p, int num_sms, int ctas_per_sm, cudaStream_t s,
+                                 const SideStream* side) {
+  return launch_by_count(
+      p, few256_render(num_sms), far256_render(num_sms), s, side,
+      [&](const RenderParams& q, cudaStream_t qs) { return launch_render_fwd256_small(q, num_sms, qs); },
+      [&](const RenderParams& q, cudaStream_t qs) {
+        if (q.loss)
+          return q.eigen ? launch_fwd256<false, true, true>(q, num_sms, ctas_per_sm, qs)
+                         : launch_fwd256<false, false, true>(q, num_sms, ctas_per_sm, qs);
+        if (q.eigen)
+          return q.lanczos ? launch_fwd256<true, true>(q, num_sms, ctas_per_sm, qs)
+                           : launch_fwd256<false, true>(q, num_sms, ctas_per_sm, qs);
+        return q.lanczos ? launch_fwd256<true, false>(q, num_sms, ctas_per_sm, qs)
+                         : launch_fwd256<false, false>(q, num_sms, ctas_per_sm, qs);
+      });
 }
 
 }  // namespace mog

@@ -121,6 +121,7 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM) render_fwd256c_kernel(Re
   float2* const w = W + f * RS;                 // the group's work row
   const int cx = (f & 1) * T;   // staged output rows, see below
   const int count = p.bucket_count[B];
+  if (count < p.bucket_min || count > p.bucket_max) return;   // the other kernel's (launch_by_count), for the whole cluster
   const int first = p.bucket_start[B];          // planned position of this bucket's first galaxy
   const unsigned char* records = p.records + (size_t)first * RECORD_BYTES;
   [[maybe_unused]] const unsigned char* records2 = COMP ? p.records2 + (size_t)first * RECORD_BYTES : nullptr;

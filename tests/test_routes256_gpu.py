@@ -229,3 +229,23 @@ def test_served_alone_and_in_a_micro_batch(gpu_renderer):
         assert np.all(np.isfinite(g0)) and np.all(np.isfinite(c0))
         np.testing.assert_array_equal(g0, g1)
         np.testing.assert_array_equal(c0, c1)
+
+
+def test_autotuning_few_galaxies_leaves_the_kernel_of_many_at_its_full_size(tables, psf0):
+    """Where the cluster kernel renders, CTAs per SM change nothing: no choice of
+    them is kept from its times, for the larger batches of the same context."""
+    import torch
+    from paper_2012_15797_gb300.renderer import Renderer, to_device
+    from workloads import mixed_galaxies
+    r = Renderer(tables, [psf0])
+    try:
+        gals = mixed_galaxies(1300, seed=94, n_psf=1)   # above the line of renders in all, 256 x 256 galaxies below both
+        assert np.count_nonzero(gals.size == 256) < 100
+        b = to_device(gals)
+        out, go = torch.empty(b.total, device="cuda"), torch.randn(b.total, device="cuda")
+        shapes = r.autotune(b, out, go, torch.empty(b.count, 6, device="cuda"), reps=1)
+        r.sync_status()
+        assert shapes[("fwd", 256)][0] == 2 and shapes[("fwd", 256)][2] == 0
+        assert shapes[("bwd", 256)][:2] == (1, 1)
+    finally:
+        r.close()
