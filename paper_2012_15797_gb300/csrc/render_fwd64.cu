@@ -17,10 +17,11 @@
 // thread (256 threads, four CTAs per SM, three barriers and twice the table and
 // component reads): 8.1k instead of 8.7k warp instructions and 1.9k instead of
 // 2.2k shared-memory wavefronts per galaxy; 100k galaxies 0.976 -> 0.935 ms, the
-// call 1.039 -> 0.998 (1.068 with the PSF spectrum read through L1, 1.018 with it in shared
+// call 1.039 -> 0.996 (1.068 with the PSF spectrum read through L1, 1.018 with it in shared
 // memory at four CTAs, 1.065 at five with the twiddles in registers, spilled),
-// the fit step of 50k 1.671 -> 1.641, 40k of an eigen-PSF 0.695 -> 0.662; with the
-// Lanczos shift (four CTAs) 30k 0.419 -> 0.421, 300 galaxies 36 -> 29 us.
+// the fit step of 50k 1.671 -> 1.638, 40k of an eigen-PSF 0.695 -> 0.658; with the
+// Lanczos shift (four CTAs) 100k 1.321 -> 1.288 (1.333 with the phases along omega
+// formed twice, for the table and for the nu = 1/2 column), 300 galaxies 36 -> 31 us.
 #include "fwd16.cuh"
 
 namespace mog {
@@ -160,13 +161,14 @@ __global__ void __launch_bounds__(THREADS, Cfg64<LZ>::CTAS_PER_SM) render_fwd64_
     const float* lzw = LZ ? p.lzw + ((size_t)first + pos) * 16 : nullptr;
     const float gx = r.x, gy = r.y;
     constexpr int NH = N / 2 + 1;
-    constexpr int t1 = NH, t2 = t1 + NH, t3 = t2 + NP;
-    for (int i = tid; i < t3 + r.nf; i += THREADS) {
+    constexpr int t1 = NH, t2 = t1 + NP;
+    for (int i = tid; i < t2 + r.nf; i += THREADS) {
       if (i < t1) {
         const int l = i;
         const float om = (float)l * INV_N;
         float2 val[2];
         const float2 phx = shift_phase(gx, 0.5f, lzw), phy = shift_phase(gy, om, LZ ? lzw + 8 : nullptr);
+        S.py[b * HALF + l] = phy;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {   // at omega and -omega; N/2 is one bin, omega = -1/2
           const bool neg = h || l == N / 2;
@@ -180,11 +182,9 @@ __global__ void __launch_bounds__(THREADS, Cfg64<LZ>::CTAS_PER_SM) render_fwd64_
         }
         S.hn[b * HALF + l] = make_float2(0.5f * (val[0].x + val[1].x), 0.5f * (val[0].y - val[1].y));
       } else if (i < t2) {
-        S.py[b * HALF + i - t1] = shift_phase(gy, (float)(i - t1) * INV_N, LZ ? lzw + 8 : nullptr);
-      } else if (i < t3) {
-        S.px[b * NP + i - t2] = shift_phase(gx, (float)(i - t2) * INV_N, lzw);
+        S.px[b * NP + i - t1] = shift_phase(gx, (float)(i - t1) * INV_N, lzw);
       } else {
-        const int c = i - t3;
+        const int c = i - t2;
         S.fc[b * KMAX + c] = make_float4(r.famp[c], r.famp[c], r.fcoef[c], r.fcoef[c]);
       }
     }
