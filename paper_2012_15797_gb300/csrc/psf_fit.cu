@@ -22,7 +22,12 @@
 // sums stand).  One warp factorises and solves, a row of the matrix per lane in
 // registers.  64 images of 64 x 64, k = 3: 49.6 -> 10.9 ms with the same bits
 // (one CTA of 256 threads per image, its chunks one after the other, thread 0
-// solving); what is left is the latency of an iteration, about 27 us.
+// solving); what is left is the latency of an iteration, about 27 us.  With more
+// images than SMs one large CTA per SM leaves it idle where a warp solves, which
+// small images do not make up for: batches of them have CTAs of 256 threads, four
+// per SM, with the same bits (3000 images of 24 x 24, k = 3: 131 ms with the first
+// form, 144 on large CTAs, 60; k = 1: 1.29, 2.23, 1.12; 40 x 40, k = 3: 158, 138,
+// 91; 1000 of 128 x 128 387, 267 on large CTAs, 297 on small ones).
 #include <cooperative_groups.h>
 
 #include "fft16.cuh"
@@ -35,23 +40,25 @@ namespace {
 constexpr int CHUNK = 256;        // pixels
 constexpr float TWO_PI_F = 6.283185307179586f;
 
-template <int K>
+// MANY: the form for batches of many small images.
+template <int K, bool MANY>
 struct FitCfg {
   static constexpr int P = 6 * K;             // parameters
   static constexpr int Q = (P + 1 + 3) & ~3;  // Jacobian row: parameters, the residual, padding
   static constexpr int NT = Q / 4;            // 4 x 4 tiles per side
   static constexpr int TILES = NT * (NT + 1) / 2;
-  static constexpr int CPS = K == 4 ? 4 : 8;  // chunks whose Jacobian rows a CTA holds
+  static constexpr int CPS = MANY ? 2 : K == 4 ? 4 : 8;  // chunks whose Jacobian rows a CTA holds
   // The pixels of several chunks are evaluated side by side (one after the
   // other by 256 threads, their latency was two thirds of an iteration).
-  static constexpr int THREADS = K == 4 ? 512 : 1024;
+  static constexpr int THREADS = MANY ? 256 : K == 4 ? 512 : 1024;
+  static constexpr int MIN_CTAS = MANY ? 4 : 1;
   static constexpr int SIDE = THREADS / CHUNK;
   static_assert(TILES * CPS <= THREADS && TILES * 16 <= THREADS, "one tile per thread, one sum per thread");
 };
 
-template <int K>
+template <int K, bool MANY>
 struct FitShared {
-  using C = FitCfg<K>;
+  using C = FitCfg<K, MANY>;
   float J[C::CPS * CHUNK * C::Q];
   float res[C::CPS * CHUNK];           // residuals at the trial point
   float part[C::CPS][C::TILES * 16];   // products of each chunk, by tile
@@ -116,16 +123,16 @@ __device__ __forceinline__ void kahan_add(float& acc, float& comp, float x) {
 template <int K>
 __device__ __forceinline__ int tiled(int i, int j) {
   const int ti = i >> 2, tj = j >> 2;
-  return (ti * FitCfg<K>::NT - ti * (ti - 1) / 2 + tj - ti) * 16 + (i & 3) * 4 + (j & 3);
+  return (ti * FitCfg<K, false>::NT - ti * (ti - 1) / 2 + tj - ti) * 16 + (i & 3) * 4 + (j & 3);
 }
 
 // The damped normal equations at S.theta (one warp of the leading CTA): with D
 // = sqrt(diag J^T J), solve (D^-1 J^T J D^-1 + lambda I) z = -D^-1 J^T r by
 // Cholesky; S.trial = theta + D^-1 z.  Lane i holds row i of the factor; every
 // entry subtracts its products in ascending order.
-template <int K>
-__device__ __forceinline__ void solve_warp(FitShared<K>& S) {
-  using C = FitCfg<K>;
+template <int K, bool MANY>
+__device__ __forceinline__ void solve_warp(FitShared<K, MANY>& S) {
+  using C = FitCfg<K, MANY>;
   constexpr int P = C::P;
   constexpr unsigned ALL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
@@ -171,16 +178,16 @@ __device__ __forceinline__ void solve_warp(FitShared<K>& S) {
   if (lane < P) S.trial[lane] = S.theta[lane] + y / Di;
 }
 
-template <int K>
-__global__ void __launch_bounds__(FitCfg<K>::THREADS) psf_fit_kernel(const float* images, int h, int w, int k, int iters,
-                                                              float* rows_out, float* chi2_out) {
-  using C = FitCfg<K>;
+template <int K, bool MANY>
+__global__ void __launch_bounds__(FitCfg<K, MANY>::THREADS, FitCfg<K, MANY>::MIN_CTAS)
+    psf_fit_kernel(const float* images, int h, int w, int k, int iters, float* rows_out, float* chi2_out) {
+  using C = FitCfg<K, MANY>;
   constexpr int P = C::P, Q = C::Q;
   extern __shared__ __align__(16) unsigned char fit_smem[];
-  FitShared<K>& S = *reinterpret_cast<FitShared<K>*>(fit_smem);
+  FitShared<K, MANY>& S = *reinterpret_cast<FitShared<K, MANY>*>(fit_smem);
   const cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
   const int rank = (int)cluster.block_rank(), ranks = (int)cluster.num_blocks();
-  FitShared<K>& S0 = *cluster.map_shared_rank(&S, 0);   // the leading CTA's
+  FitShared<K, MANY>& S0 = *cluster.map_shared_rank(&S, 0);   // the leading CTA's
   const bool lead = rank == 0;
   const int tid = threadIdx.x, px = tid % CHUNK, image = blockIdx.x / ranks;
   const float* img = images + (size_t)image * h * w;
@@ -350,7 +357,7 @@ __global__ void __launch_bounds__(FitCfg<K>::THREADS) psf_fit_kernel(const float
     }
     if (lead && tid < 32) {
       __syncwarp();
-      solve_warp<K>(S);
+      solve_warp<K, MANY>(S);
     }
     cluster.sync();   // the trial point is there
   }
@@ -382,25 +389,17 @@ __global__ void __launch_bounds__(FitCfg<K>::THREADS) psf_fit_kernel(const float
   cluster.sync();   // no CTA ends while another may read its shared memory
 }
 
-template <int K>
-cudaError_t launch_fit(const float* images, int count, int h, int w, int iters, float* rows, float* chi2,
-                       cudaStream_t s) {
-  using C = FitCfg<K>;
-  const int occ = kernel_occupancy(reinterpret_cast<const void*>(psf_fit_kernel<K>), C::THREADS, sizeof(FitShared<K>));
-  if (occ < 0) return cudaErrorInvalidConfiguration;
-  int device = 0, sms = 0;
-  cudaError_t e = cudaGetDevice(&device);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-  if (e != cudaSuccess) return e;
-  // As many CTAs per image (1, 2, 4 or 8) as the SMs hold at once and the
-  // image has chunks for.
-  const int64_t steps = ((int64_t)h * w + CHUNK * C::CPS - 1) / (CHUNK * C::CPS);
-  int cl = 1;
-  while (cl < 8 && (int64_t)count * cl * 2 <= sms && cl < steps) cl *= 2;
+template <int K, bool MANY>
+cudaError_t launch_fit_as(const float* images, int count, int h, int w, int iters, float* rows, float* chi2, int cl,
+                          cudaStream_t s) {
+  using C = FitCfg<K, MANY>;
+  constexpr size_t SMEM = sizeof(FitShared<K, MANY>);
+  if (kernel_occupancy(reinterpret_cast<const void*>(psf_fit_kernel<K, MANY>), C::THREADS, SMEM) < 0)
+    return cudaErrorInvalidConfiguration;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)count * cl);
   cfg.blockDim = dim3(C::THREADS);
-  cfg.dynamicSmemBytes = sizeof(FitShared<K>);
+  cfg.dynamicSmemBytes = SMEM;
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -408,7 +407,34 @@ cudaError_t launch_fit(const float* images, int count, int h, int w, int iters, 
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, psf_fit_kernel<K>, images, h, w, K, iters, rows, chi2);
+  return cudaLaunchKernelEx(&cfg, psf_fit_kernel<K, MANY>, images, h, w, K, iters, rows, chi2);
+}
+
+template <int K>
+cudaError_t launch_fit(const float* images, int count, int h, int w, int iters, float* rows, float* chi2,
+                       cudaStream_t s) {
+  int device = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&device);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+  if (e != cudaSuccess) return e;
+  const int64_t chunks = ((int64_t)h * w + CHUNK - 1) / CHUNK;
+  // Many small images: CTAs of 256 threads, four per SM, so that one computes
+  // while another waits or solves (see the header).  From three images per SM on
+  // (608 of 24 x 24, k = 3: 12.3 ms against 31; 304 of 40 x 40 20.7 against 19.1);
+  // larger images keep the large CTAs, whose iterations are shorter.  So do most
+  // fits with two components, where some images take many more iterations than
+  // the others and the call waits for them (3000 of 40 x 40: 24 ms against 20.5).
+  if constexpr (K < 4) {
+    if (count > (K == 2 ? 12 : 3) * sms && (chunks <= (K == 2 ? 5 : 24) || (K == 1 && count > 12 * sms)))
+      return launch_fit_as<K, true>(images, count, h, w, iters, rows, chi2, 1, s);
+  }
+  // As many CTAs per image (1, 2, 4 or 8) as the SMs hold at once and the
+  // image has chunks for.
+  constexpr int CPS = FitCfg<K, false>::CPS;
+  const int64_t steps = (chunks + CPS - 1) / CPS;
+  int cl = 1;
+  while (cl < 8 && (int64_t)count * cl * 2 <= sms && cl < steps) cl *= 2;
+  return launch_fit_as<K, false>(images, count, h, w, iters, rows, chi2, cl, s);
 }
 
 }  // namespace
