@@ -412,10 +412,9 @@ mog_status mog_render_backward_ex(mog_ctx* ctx, const mog_batch* batch, const fl
  * galaxies) with CUDA events, `reps` renders per choice, and keeps the
  * fastest in the context for later calls (schedules 1 and 2 apply to the
  * plain render; the Lanczos and eigen-PSF variants keep the first).  256 x 256
- * galaxies have a second kernel for small numbers of them (up to 3000, 1500 with
- * the Lanczos shift or composites; the adjoint two per SM), with the same
- * results: it takes no CTAs per SM, and its adjoint no chunk, so those are not
- * tuned where it runs.  With
+ * galaxies have a second kernel for small numbers of them (up to 8 per SM; the
+ * adjoint 0.75, with the Lanczos shift 1.5), with the same results: it takes no
+ * CTAs per SM, and its adjoint no chunk, so those are not tuned where it runs.  With
  * several sizes in the batch it then times the whole render with the size
  * kernels forked onto parallel streams and one after the other, and keeps the
  * faster.  With non-null grad_out and grad_params the adjoint's launch shapes
