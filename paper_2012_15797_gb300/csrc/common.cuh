@@ -162,7 +162,8 @@ __device__ __forceinline__ void dft_r(float2* v) {
 // pass is always radix 8 on the thread's 8 values): V = 0: 32 = 8*4,
 // 64 = 8*8, 128 = 8*8*2, 256 = 8*8*4; V = 1: 32 = 8*2*2, 64 = 8*4*2,
 // 128 = 8*4*4, 256 = 8*4*8 (the autotuner picks per patch side; the 256 x 256
-// render has its own transforms, fft16.cuh, under both numbers).  A pass of radix R with current
+// kernels have their own transforms, fft16.cuh, under both numbers, so that no
+// kernel takes its second schedule, and its first only the PSFs' spectra).  A pass of radix R with current
 // sub-length Ns: butterfly b reads x[b + m N/R] (m < R), multiplies by
 // w_{Ns R}^{m (b mod Ns)}, takes an R-point DFT and writes
 // x'[(b / Ns) Ns R + (b mod Ns) + m Ns].  Thread j owns butterflies

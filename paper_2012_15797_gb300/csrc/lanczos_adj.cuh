@@ -8,12 +8,12 @@
 // through d alone (n is piecewise constant), so for an upstream gradient g
 //   dL/dtheta = <Lz^T g, dI/dtheta>          (flux, log r_e, e1, e2, Sersic n)
 //   dL/dx     = <(dLz/d d_x)^T g, I>,
-// and likewise dL/dy.  The adjoint kernels (render_bwd.cu, render_bwd256.cu)
-// take one forward transform of g for all of them: on the spectrum the
-// transposed convolutions are multiplications by the conjugate responses of w
-// and of the slopes w' = dw/dd, folded into the phase tables; for the
-// real-space terms they are formed from the patch where it is read.  Measured
-// on 10k 64 x 64 galaxies: 0.321 ms a call; a kernel that wrote the three
+// and likewise dL/dy.  The adjoint kernels (render_bwd*.cu) take one forward
+// transform of g for all of them: on the spectrum the transposed convolutions
+// are multiplications by the conjugate responses of w and of the slopes w' =
+// dw/dd, folded into the phase tables; for the real-space terms they are formed
+// from the patch where it is read.  Measured
+// on 10k 64 x 64 galaxies: 0.335 ms a call; a kernel that wrote the three
 // convolved patches, an adjoint pass over each and a synchronisation to size
 // them took 1.453 ms (the plain adjoint of one pass takes 0.24 ms).
 #pragma once

@@ -15,8 +15,8 @@
 // Issue slots, shared memory and latency at 20 warps per SM bound it (issue 65%,
 // l1tex 70%).  Against 8 values per
 // thread (256 threads, four CTAs per SM, three barriers and twice the table and
-// component reads): 8.1k instead of 8.7k warp instructions and 1.9k instead of
-// 2.2k shared-memory wavefronts per galaxy; 100k galaxies 0.976 -> 0.935 ms, the
+// component reads): 7.9k instead of 8.7k warp instructions and 1.9k instead of
+// 2.2k shared-memory wavefronts per galaxy; 100k galaxies 0.976 -> 0.930 ms, the
 // call 1.039 -> 0.996 (1.068 with the PSF spectrum read through L1, 1.018 with it in shared
 // memory at four CTAs, 1.065 at five with the twiddles in registers, spilled),
 // the fit step of 50k 1.671 -> 1.638, 40k of an eigen-PSF 0.695 -> 0.658; with the
